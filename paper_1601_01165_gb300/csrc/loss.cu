@@ -80,6 +80,14 @@ __device__ __forceinline__ DF df_add(DF a, DF b) {
   return fast_two_sum(u.h, __fadd_rn(u.l, t.l));
 }
 
+// The same for the sums below, where a.l + b.l needs no exact error: two
+// operations instead of nine.  The result is within 2^-47 (|a| + |b|), and
+// exact wherever |a.l + b.l| fits 24 bits of the operands' common unit.
+__device__ __forceinline__ DF df_add_fast(DF a, DF b) {
+  const DF s = two_sum(a.h, b.h);
+  return fast_two_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+
 // d * d for a two-float d, as a two-float (the low part's square is dropped)
 __device__ __forceinline__ DF df_sqr(DF d) {
   const float p = __fmul_rn(d.h, d.h);
@@ -97,100 +105,159 @@ __device__ __forceinline__ double df_value(DF a) { return (double)a.h + (double)
 // a > b for normalised two-floats
 __device__ __forceinline__ bool df_gt(DF a, DF b) { return a.h > b.h || (a.h == b.h && a.l > b.l); }
 
-// The boxcar starting at t as a two-float (exact while the 8 values' nonzero
-// magnitudes lie within a factor of about 2^21: 48 bits hold the sum of eight
-// 24-bit significands spread that far).
-__device__ __forceinline__ DF boxcar_df(const float* row, int64_t t) {
-  DF b{0.0f, 0.0f};
+// The boxcars of a thread's K consecutive starts, from x[0 .. K + 7): pairs,
+// fours, eights, each shared by the boxcars that need it (one add of floats
+// and two of two-floats per start, against eight adds for a boxcar summed by
+// itself).  Exact while the values' nonzero magnitudes lie within a factor of
+// about 2^21: 48 bits hold the sum of eight 24-bit significands spread that far.
+// visit(k, boxcar) in order of k.
+template <int K, typename F>
+__device__ __forceinline__ void boxcars(const float* x, F visit) {
+  DF p2[6];  // pairs starting at the last six samples, then fours likewise
+  DF p4[4];
 #pragma unroll
-  for (int k = 0; k < kBox; ++k) b = df_add_f(b, __ldg(row + t + k));
-  return b;
+  for (int u = 0; u < K + 6; ++u) {
+    const DF two = two_sum(x[u], x[u + 1]);
+    if (u >= 2) {
+      const DF four = df_add_fast(p2[(u - 2) % 6], two);  // starts at u - 2
+      if (u >= 6) visit(u - 6, df_add_fast(p4[(u - 6) % 4], four));
+      p4[(u - 2) % 4] = four;
+    }
+    p2[u % 6] = two;
+  }
 }
 
-// One block per row: mean, sd, best S/N and where it is.  Thread j takes
-// the boxcar starts j, j + NT, ... (coalesced loads; each boxcar summed from
-// its 8 values in two-float arithmetic, exact while their nonzero magnitudes
-// lie within a factor of about 2^21, so b equals the direct 8-term sum and
-// its double value).  Pass 1: the sum of b and the largest b (first t); pass 2: the
-// variance about the mean (each thread's sums in two-float, the block's in
-// double); the best S/N is (b_max - mean) / sd in double.  S/N is monotonic
-// in b, so the first maximum of S/N lies among the starts whose b is within
-// rounding of b_max; pass 3 takes the first start before that t whose S/N
-// equals the best (a different t only when two sums round to one S/N).
-template <int NT>
+// One block per row: mean, sd, best S/N and where it is; with ZERO the block
+// also clears the row of the gradient while it computes.
+//
+// Instruction issue bounds it (75 % of the slots; about 120 instructions a sample, where
+// reading and clearing a 2048 x 20,000 block of 164 MB take 24 us each), so a
+// row is passed over twice with as little as each needs:
+//  1. the sum of the samples, which gives the boxcars' (a sample counts in
+//     eight of them, at the row's ends in fewer);
+//  2. from tiles of the row in shared memory, each thread's K consecutive
+//     boxcars: the squares about the mean and the largest boxcar (K odd: the
+//     lanes' reads hit distinct banks).
+// Threads sum in two-float arithmetic, the block in double.  S/N is monotonic
+// in the boxcar, so the best S/N is (b_max - mean) / sd, and the first start
+// with that S/N lies among those whose boxcar is within rounding of b_max:
+// only a thread that has another boxcar that close goes over its starts again
+// (a different start only when two sums round to one S/N).
+// 2048 x 20,000 with the gradient: the whole call 204 us, nearly all of it this
+// kernel (before: 493, every boxcar summed by itself in each of three passes,
+// the clearing after them, and 0.1 ms for the one row of the gradient).
+template <int NT, int K, bool ZERO>
 __global__ void __launch_bounds__(NT) snr_rows_kernel(const float* __restrict__ x, int64_t stride, int64_t n_cols,
-                                                      RowStat* __restrict__ stats) {
+                                                      RowStat* __restrict__ stats, float* __restrict__ grad,
+                                                      int64_t grad_stride) {
+  constexpr int TILE = NT * K;
+  __shared__ float tile[TILE + kBox - 1];
   __shared__ double red[NT];
-  __shared__ double zbest[NT];
   __shared__ int64_t tbest[NT];
-  const int i = blockIdx.x;
+  const int i = blockIdx.x, tid = threadIdx.x;
   const float* row = x + (int64_t)i * stride;
   const int64_t nb = n_cols - kBox + 1;
 
-  // pass 1: sum and largest boxcar
-  DF s{0.0f, 0.0f}, bmax{-FLT_MAX, 0.0f};
-  int64_t tmax = -1;
-  for (int64_t t = threadIdx.x; t < nb; t += NT) {
-    const DF b = boxcar_df(row, t);
-    s = df_add(s, b);
-    if (tmax < 0 || df_gt(b, bmax)) {  // t increases, so the first maximum is kept
-      bmax = b;
-      tmax = t;
-    }
+  // pass 1: the sum of the boxcars (a sample u is in min(u + 1, 8, n_cols - u, nb) of them)
+  DF s4[4] = {};
+  int64_t u = tid;
+  for (; u + 3 * NT < n_cols; u += 4 * NT) {
+    float v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = __ldg(row + u + k * NT);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s4[k] = df_add_f(s4[k], v[k]);
   }
-  const double mean = block_sum<NT>(df_value(s), red) / (double)nb;
-  zbest[threadIdx.x] = df_value(bmax);
-  tbest[threadIdx.x] = tmax;
+  for (; u < n_cols; u += NT) s4[0] = df_add_f(s4[0], __ldg(row + u));
+  double sum = (double)kBox * df_value(df_add(df_add(s4[0], s4[1]), df_add(s4[2], s4[3])));
+  for (int64_t e = tid; e < 2 * (kBox - 1); e += NT) {  // the ends: count the missing ones off
+    const int64_t at = e < kBox - 1 ? e : n_cols - 1 - (e - (kBox - 1));
+    const int64_t lo = min(at + 1, (int64_t)kBox), hi = min(n_cols - at, nb);
+    // (a short row's two ends may meet: each sample once)
+    if (at >= 0 && (e < kBox - 1 ? at < n_cols : at >= kBox - 1)) sum -= (double)(kBox - min(lo, hi)) * (double)__ldg(row + at);
+  }
+  const double mean = block_sum<NT>(sum, red) / (double)nb;
+
+  // pass 2: squares about the mean, and the largest boxcar of each thread (its first)
+  const DF neg_mean = df_of(-mean);
+  DF v{0.0f, 0.0f}, bmax{-FLT_MAX, 0.0f}, before{-FLT_MAX, 0.0f};  // `before`: the largest at earlier starts
+  int at = -1;     // its place among this thread's starts, tile by tile
+  int first = 0;   // the tile's first place
+  for (int64_t base = 0; base < nb; base += TILE, first += K) {
+    const int64_t len = min((int64_t)(TILE + kBox - 1), n_cols - base);
+    for (int64_t k = tid; k < len; k += NT) tile[k] = __ldg(row + base + k);
+    if constexpr (ZERO) {
+      // (the last tile also clears the samples past the last start)
+      float* gr = grad + (int64_t)i * grad_stride + base;
+      const int64_t glen = base + TILE < nb ? (int64_t)TILE : n_cols - base;
+      for (int64_t k = tid; k < glen; k += NT) gr[k] = 0.0f;
+    }
+    __syncthreads();
+    const int64_t t0 = base + (int64_t)tid * K;
+    const int n = (int)max((int64_t)0, min((int64_t)K, nb - t0));
+    auto visit = [&](int k, DF b) {
+      if (k < n) {
+        const DF c = two_sum(b.h, neg_mean.h);
+        const DF d = fast_two_sum(c.h, __fadd_rn(c.l, __fadd_rn(b.l, neg_mean.l)));
+        v = df_add_fast(v, df_sqr(d));
+        if (at < 0 || df_gt(b, bmax)) {  // t increases, so the first maximum is kept
+          before = bmax;
+          bmax = b;
+          at = first + k;
+        }
+      }
+    };
+    if (n > 0) boxcars<K>(tile + tid * K, visit);
+    __syncthreads();
+  }
+  const double sd = sqrt(block_sum<NT>(df_value(v), red) / (double)nb);
+
+  // the row's largest boxcar, its first start
+  const double mine = df_value(bmax);
+  const int64_t tmax = at < 0 ? -1 : (int64_t)(at / K) * TILE + (int64_t)tid * K + at % K;
+  red[tid] = mine;
+  tbest[tid] = tmax;
   __syncthreads();
   for (int h = NT / 2; h > 0; h >>= 1) {
-    if ((int)threadIdx.x < h) {
-      const double bo = zbest[threadIdx.x + h];
-      const int64_t to = tbest[threadIdx.x + h];
-      if (to >= 0 && (tbest[threadIdx.x] < 0 || bo > zbest[threadIdx.x] ||
-                      (bo == zbest[threadIdx.x] && to < tbest[threadIdx.x]))) {
-        zbest[threadIdx.x] = bo;
-        tbest[threadIdx.x] = to;
+    if (tid < h) {
+      const double bo = red[tid + h];
+      const int64_t to = tbest[tid + h];
+      if (to >= 0 && (tbest[tid] < 0 || bo > red[tid] || (bo == red[tid] && to < tbest[tid]))) {
+        red[tid] = bo;
+        tbest[tid] = to;
       }
     }
     __syncthreads();
   }
-  const double b_top = zbest[0];
+  const double b_top = red[0];
   const int64_t t_top = tbest[0];
   __syncthreads();
-
-  // pass 2: variance about the mean
-  const DF neg_mean = df_of(-mean);
-  DF v{0.0f, 0.0f};
-  for (int64_t t = threadIdx.x; t < nb; t += NT) v = df_add(v, df_sqr(df_add(boxcar_df(row, t), neg_mean)));
-  const double sd = sqrt(block_sum<NT>(df_value(v), red) / (double)nb);
   if (!(sd > 0.0)) {
-    if (threadIdx.x == 0) stats[i] = RowStat{-DBL_MAX, mean, sd, -1};
+    if (tid == 0) stats[i] = RowStat{-DBL_MAX, mean, sd, -1};
     return;
   }
   const double z_top = (b_top - mean) / sd;
 
-  // pass 3: the first start before t_top with the same S/N, if any
+  // the first start with the same S/N, if it is before t_top
   const double b_cut = b_top - 1e-12 * (fabs(b_top - mean) + fabs(b_top));
   int64_t tf = t_top;
-  // below cut_f (two float steps under b_cut) a two-float value is surely below b_cut
-  const float cut_f = nextafterf(nextafterf((float)b_cut, -FLT_MAX), -FLT_MAX);
-  for (int64_t t = threadIdx.x; t < t_top; t += NT) {
-    const DF b = boxcar_df(row, t);
-    if (b.h >= cut_f) {
-      const double bd = df_value(b);
-      if (bd >= b_cut && (bd - mean) / sd == z_top) {
-        tf = t;
-        break;
+  if (tmax >= 0 && (tmax == t_top ? df_value(before) : mine) >= b_cut) {
+    for (int64_t base = 0; base < t_top && tf == t_top; base += TILE)
+      for (int64_t t = base + (int64_t)tid * K; t < min(base + (int64_t)(tid + 1) * K, t_top); ++t) {
+        const double bd = boxcar(row, t);
+        if (bd >= b_cut && (bd - mean) / sd == z_top) {
+          tf = t;
+          break;
+        }
       }
-    }
   }
-  tbest[threadIdx.x] = tf;
+  tbest[tid] = tf;
   __syncthreads();
   for (int h = NT / 2; h > 0; h >>= 1) {
-    if ((int)threadIdx.x < h) tbest[threadIdx.x] = min(tbest[threadIdx.x], tbest[threadIdx.x + h]);
+    if (tid < h) tbest[tid] = min(tbest[tid], tbest[tid + h]);
     __syncthreads();
   }
-  if (threadIdx.x == 0) stats[i] = RowStat{z_top, mean, sd, tbest[0]};
+  if (tid == 0) stats[i] = RowStat{z_top, mean, sd, tbest[0]};
 }
 
 // One block: the best row (first on ties) -> result.
@@ -241,41 +308,50 @@ __global__ void __launch_bounds__(NT) snr_pick_kernel(const RowStat* __restrict_
   }
 }
 
-// d loss / d x for the best row (the other rows were zeroed by the caller).
-__global__ void snr_grad_kernel(const float* __restrict__ x, int64_t stride, int64_t n_cols,
-                                const dd_snr_result* __restrict__ result, float* __restrict__ grad,
-                                int64_t grad_stride) {
+// d loss / d x for the best row (the rows kernel cleared all).  Double divisions
+// and each boxcar eight times over made this one row cost 0.1 ms; every start's
+// term is now made once, by multiplications, and shared through the block.
+template <int NT>
+__global__ void __launch_bounds__(NT) snr_grad_kernel(const float* __restrict__ x, int64_t stride, int64_t n_cols,
+                                                      const dd_snr_result* __restrict__ result,
+                                                      float* __restrict__ grad, int64_t grad_stride) {
+  __shared__ double db[NT + kBox - 1];  // d snr / d b of the starts [u0 - 7, u0 + NT)
+  if (!result->valid) return;
   const dd_snr_result r = *result;
-  if (!r.valid) return;
-  const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (u >= n_cols) return;
+  const int64_t u0 = (int64_t)blockIdx.x * NT;
   const float* row = x + (int64_t)r.best_row * stride;
   const int64_t nb = n_cols - kBox + 1;
-  double acc = 0.0;
-  const int64_t t_lo = u - (kBox - 1) > 0 ? u - (kBox - 1) : 0;
-  const int64_t t_hi = u < nb - 1 ? u : nb - 1;
-  for (int64_t t = t_lo; t <= t_hi; ++t) {
-    const double z = (boxcar(row, t) - r.mean) / r.std;
-    acc += ((t == r.best_t ? 1.0 : 0.0) - 1.0 / (double)nb) / r.std - r.snr * z / ((double)nb * r.std);
+  const double inv_sd = 1.0 / r.std, inv_nb = 1.0 / (double)nb;
+  for (int k = threadIdx.x; k < NT + kBox - 1; k += NT) {
+    const int64_t t = u0 - (kBox - 1) + k;
+    double v = 0.0;
+    if (t >= 0 && t < nb) {
+      const double z = (boxcar(row, t) - r.mean) * inv_sd;
+      v = ((t == r.best_t ? 1.0 : 0.0) - inv_nb * (1.0 + r.snr * z)) * inv_sd;
+    }
+    db[k] = v;
   }
+  __syncthreads();
+  const int64_t u = u0 + threadIdx.x;
+  if (u >= n_cols) return;
+  double acc = 0.0;
+#pragma unroll
+  for (int k = 0; k < kBox; ++k) acc += db[threadIdx.x + k];
   grad[(int64_t)r.best_row * grad_stride + u] = (float)(-acc);
 }
 
 dd_status boxcar_snr_launch(const char* who, const float* x, int64_t row_stride, int32_t n_rows, int64_t n_cols,
                             dd_snr_result* result, float* grad, int64_t grad_stride, cudaStream_t s, void* scratch) {
-  constexpr int NT = 256;
+  constexpr int NT = 256, K = 15;
   RowStat* stats = static_cast<RowStat*>(scratch);
-  snr_rows_kernel<NT><<<n_rows, NT, 0, s>>>(x, row_stride, n_cols, stats);
+  if (grad)
+    snr_rows_kernel<NT, K, true><<<n_rows, NT, 0, s>>>(x, row_stride, n_cols, stats, grad, grad_stride);
+  else
+    snr_rows_kernel<NT, K, false><<<n_rows, NT, 0, s>>>(x, row_stride, n_cols, stats, nullptr, 0);
   snr_pick_kernel<NT><<<1, NT, 0, s>>>(stats, n_rows, result);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && grad) {
-    e = cudaMemset2DAsync(grad, grad_stride * sizeof(float), 0, n_cols * sizeof(float), n_rows, s);
-    if (e == cudaSuccess) {
-      snr_grad_kernel<<<(unsigned)((n_cols + 255) / 256), 256, 0, s>>>(x, row_stride, n_cols, result, grad,
-                                                                         grad_stride);
-      e = cudaGetLastError();
-    }
-  }
+  if (grad)
+    snr_grad_kernel<NT><<<(unsigned)((n_cols + NT - 1) / NT), NT, 0, s>>>(x, row_stride, n_cols, result, grad, grad_stride);
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return set_error(DD_ERR_CUDA, "%s: launch: %s (%s)", who, cudaGetErrorString(e),
                                          cudaGetErrorName(e));
   return DD_OK;
