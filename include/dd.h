@@ -242,8 +242,10 @@ dd_status dd_forward_host(dd_plan_t plan, const void* host_in, int64_t in_row_st
  * on a float plan that offers the 9-trial Tensor-Memory kernel and
  * an `in` that kernel takes (16-byte aligned rows of dd_plan_in_stride), it
  * is computed directly on that kernel's tiles (about twice the forward's
- * time); otherwise from the transpose.  The two ways sum in different orders
- * (both within the float tolerance of the exact result).  Either uses
+ * time), or, where at most eight rows of grad_out (and half of them) have a
+ * nonzero and every sample of `in` is finite, from these rows alone (a few
+ * percent of it); otherwise from the transpose.  These ways sum in different
+ * orders (all within the float tolerance of the exact result).  They use
  * scratch buffers the plan allocates on first use.
  * Errors: DD_ERR_UNSUPPORTED on a uint8 plan, DD_ERR_ARG if both outputs are
  * NULL or grad_w is requested without `in`, DD_ERR_SHAPE, DD_ERR_NOMEM,

@@ -55,20 +55,135 @@ static dd_status adjoint_plan(dd_plan_s* p, dd_plan_s** out) {
 }
 
 // grad_w[c] = sum_u in[c][u] * g[c][u]: one block per channel, double sums,
-// fixed reduction tree.
-__global__ void __launch_bounds__(256) wgrad_dot_kernel(const float* __restrict__ in, int64_t in_stride,
-                                                        const float* __restrict__ g, int64_t g_stride, int64_t n,
+// fixed reduction tree.  With SCALE the same pass leaves w[c] * g[c][u] in g
+// (the input gradient), which otherwise takes another reading of it.
+template <bool SCALE>
+__global__ void __launch_bounds__(256) wgrad_dot_kernel(const float* __restrict__ in, int64_t in_stride, float* g,
+                                                        int64_t g_stride, int64_t n, const float* __restrict__ w,
                                                         float* __restrict__ grad_w) {
   const int c = blockIdx.x;
   const float* a = in + (int64_t)c * in_stride;
-  const float* b = g + (int64_t)c * g_stride;
+  float* b = g + (int64_t)c * g_stride;
+  const float wc = SCALE ? __ldg(w + c) : 1.0f;
   double acc = 0.0;
-  for (int64_t u = threadIdx.x; u < n; u += blockDim.x) acc += (double)__ldg(a + u) * (double)__ldg(b + u);
+  int64_t u = threadIdx.x;
+  for (; u + 768 < n; u += 1024) {
+    float x[4], y[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = __ldg(a + u + 256 * k), y[k] = b[u + 256 * k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      acc += (double)x[k] * (double)y[k];
+      if constexpr (SCALE) b[u + 256 * k] = y[k] * wc;
+    }
+  }
+  for (; u < n; u += 256) {
+    const float y = b[u];
+    acc += (double)__ldg(a + u) * (double)y;
+    if constexpr (SCALE) b[u] = y * wc;
+  }
   __shared__ double red[256];
   red[threadIdx.x] = acc;
   __syncthreads();
   for (int s = 128; s > 0; s >>= 1) {
     if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) grad_w[c] = (float)red[0];
+}
+
+// ------------------------------------------ weight gradient of few rows
+// The detection loss has a gradient in one row only, and so has any loss that
+// looks at single trials.  The tile kernel multiplies the other rows' zeros
+// all the same (2048 trials: 4.6 ms for what one row's products give in 0.02),
+// so the rows with a nonzero are listed first, and if there are at most
+// kFewRows of them, and they are at most half of all, wgrad_rows_kernel does
+// the products of those rows alone.  A zero times an infinity or NaN of the
+// input is not zero: with such a sample in the input the tiles do it all.
+// The choice is made on the device, by kernels that cost 0.02 ms (a dense
+// gradient is given up at its rows' first samples).
+constexpr int kFewRows = 8;
+
+// any[i] = row i of g has a nonzero (a NaN is one)
+__global__ void __launch_bounds__(256) wgrad_scan_kernel(const float* __restrict__ g, int64_t stride, int64_t n,
+                                                         int* __restrict__ any) {
+  const float* row = g + (int64_t)blockIdx.x * stride;
+  int found = 0;
+  for (int64_t base = 0; base < n && !found; base += 256 * 8) {
+    bool nz = false;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int64_t t = base + 256 * k + threadIdx.x;
+      if (t < n) nz |= !(__ldg(row + t) == 0.0f);
+    }
+    found = __syncthreads_or(nz);
+  }
+  if (threadIdx.x == 0) any[blockIdx.x] = found;
+}
+
+// One block: few.rows, few.list (ascending) and few.use.
+__global__ void __launch_bounds__(1024) wgrad_list_kernel(const int* __restrict__ any, int n_rows, WgradFew* few) {
+  __shared__ int cnt[1024];
+  const int per = (n_rows + 1023) / 1024, i0 = (int)threadIdx.x * per, i1 = min(n_rows, i0 + per);
+  int mine = 0;
+  for (int i = i0; i < i1; ++i) mine += any[i];
+  cnt[threadIdx.x] = mine;
+  __syncthreads();
+  for (int o = 1; o < 1024; o *= 2) {
+    const int v = (int)threadIdx.x >= o ? cnt[threadIdx.x - o] : 0;
+    __syncthreads();
+    cnt[threadIdx.x] += v;
+    __syncthreads();
+  }
+  const int total = cnt[1023];
+  const bool use = total <= kFewRows && 2 * total <= n_rows;
+  if (use) {
+    int at = cnt[threadIdx.x] - mine;
+    for (int i = i0; i < i1; ++i)
+      if (any[i]) few->list[at++] = i;
+  }
+  if (threadIdx.x == 0) {
+    few->rows = total;
+    few->use = use ? 1 : 0;
+  }
+}
+
+// few.use = 0 if a sample of the input is not finite.
+__global__ void __launch_bounds__(256) wgrad_finite_kernel(const float* __restrict__ in, int64_t stride, int64_t n,
+                                                           WgradFew* few) {
+  if (!few->use) return;
+  const float* row = in + (int64_t)blockIdx.x * stride;
+  bool bad = false;
+  for (int64_t t = threadIdx.x; t < n; t += 256) bad |= !(fabsf(__ldg(row + t)) <= 3.402823466e38f);
+  if (__syncthreads_or(bad) && threadIdx.x == 0) few->use = 0;
+}
+
+// grad_w[c] of the listed rows, one block per channel: four short float chains
+// a thread and row, then double; a fixed order.
+__global__ void __launch_bounds__(256) wgrad_rows_kernel(const float* __restrict__ g, int64_t g_stride,
+                                                         const float* __restrict__ in, int64_t in_stride,
+                                                         const int32_t* __restrict__ delays, int C, int64_t n,
+                                                         const WgradFew* __restrict__ few, float* __restrict__ grad_w) {
+  if (!few->use) return;
+  const int c = blockIdx.x, rows = few->rows;
+  double sum = 0.0;
+  for (int r = 0; r < rows; ++r) {
+    const int i = few->list[r];
+    const float* a = g + (int64_t)i * g_stride;
+    const float* b = in + (int64_t)c * in_stride + delays[(int64_t)i * C + c];
+    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    int64_t t = threadIdx.x;
+    for (; t + 768 < n; t += 1024)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) s[k] = fmaf(__ldg(a + t + 256 * k), __ldg(b + t + 256 * k), s[k]);
+    for (; t < n; t += 256) s[0] = fmaf(__ldg(a + t), __ldg(b + t), s[0]);
+    sum += ((double)s[0] + (double)s[1]) + ((double)s[2] + (double)s[3]);
+  }
+  __shared__ double red[256];
+  red[threadIdx.x] = sum;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
     __syncthreads();
   }
   if (threadIdx.x == 0) grad_w[c] = (float)red[0];
@@ -110,16 +225,27 @@ extern "C" dd_status dd_adjoint(dd_plan_t plan, const float* grad_out, int64_t g
     // (12 partial sums per channel and tile: past 1 GiB of them, as for very
     // long outputs, the transposed path below needs less memory)
     if (n > 0 && n <= ((int64_t)1 << 28)) {
+      // (the partial sums, then what lists the rows)
+      const size_t bytes = (size_t)n * sizeof(float) + sizeof(WgradFew) + (size_t)plan->n_dm * sizeof(int);
       if (plan->adj_wpart_floats < n) {
         cudaFree(plan->adj_wpart);
         plan->adj_wpart_floats = 0;
-        if (cudaMalloc(&plan->adj_wpart, (size_t)n * sizeof(float)) != cudaSuccess) {
+        if (cudaMalloc(&plan->adj_wpart, bytes) != cudaSuccess) {
           plan->adj_wpart = nullptr;
           return set_error(DD_ERR_NOMEM, "dd_adjoint: cannot allocate %lld floats of partial sums", (long long)n);
         }
         plan->adj_wpart_floats = n;
       }
-      const cudaError_t e = launch_tmw9_wgrad(a, grad_out, go_row_stride, plan->adj_wpart, grad_w, s);
+      // (n is a multiple of 12: the structure after it is aligned to 16 bytes)
+      WgradFew* few = reinterpret_cast<WgradFew*>(plan->adj_wpart + plan->adj_wpart_floats);
+      int* any = reinterpret_cast<int*>(few + 1);
+      wgrad_scan_kernel<<<plan->n_dm, 256, 0, s>>>(grad_out, go_row_stride, plan->n_out, any);
+      wgrad_list_kernel<<<1, 1024, 0, s>>>(any, plan->n_dm, few);
+      wgrad_finite_kernel<<<plan->C, 256, 0, s>>>(in, in_row_stride, plan->n_in, few);
+      wgrad_rows_kernel<<<plan->C, 256, 0, s>>>(grad_out, go_row_stride, in, in_row_stride, plan->d_delays, plan->C,
+                                                plan->n_out, few, grad_w);
+      cudaError_t e = cudaGetLastError();
+      if (e == cudaSuccess) e = launch_tmw9_wgrad(a, grad_out, go_row_stride, plan->adj_wpart, few, grad_w, s);
       if (e != cudaSuccess) return set_cuda_error("dd_adjoint: weight gradient", e);
       return DD_OK;
     }
@@ -164,10 +290,12 @@ extern "C" dd_status dd_adjoint(dd_plan_t plan, const float* grad_out, int64_t g
   st = forward_device(q, plan->adj_pad, plan->adj_pad_stride, nullptr, g, g_stride, s, -1);
   if (st != DD_OK) return st;
   if (grad_w) {
-    wgrad_dot_kernel<<<plan->C, 256, 0, s>>>(in, in_row_stride, g, g_stride, plan->n_in, grad_w);
+    if (grad_in && w)
+      wgrad_dot_kernel<true><<<plan->C, 256, 0, s>>>(in, in_row_stride, g, g_stride, plan->n_in, w, grad_w);
+    else
+      wgrad_dot_kernel<false><<<plan->C, 256, 0, s>>>(in, in_row_stride, g, g_stride, plan->n_in, nullptr, grad_w);
     if ((e = cudaGetLastError()) != cudaSuccess) return set_cuda_error("dd_adjoint: weight gradient", e);
-  }
-  if (grad_in && w) {
+  } else if (grad_in && w) {
     dim3 grid((unsigned)std::min<int64_t>((plan->n_in + 255) / 256, 1024), (unsigned)plan->C);
     scale_rows_kernel<<<grid, 256, 0, s>>>(grad_in, gi_row_stride, plan->n_in, w);
     if ((e = cudaGetLastError()) != cudaSuccess) return set_cuda_error("dd_adjoint: weights", e);

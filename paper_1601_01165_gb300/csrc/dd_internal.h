@@ -169,12 +169,19 @@ cudaError_t launch_persistent(const TileConfig& cfg, dd_dtype dtype, const Batch
                               cudaStream_t s);
 size_t tmw9_views_bytes();
 bool tmw9_encode_views(const FwdArgs& a, void* out);
+// The rows of grad_out that have a nonzero, if few (adjoint.cu): with `use`
+// the weight gradient has been computed from them and the tiles do nothing.
+struct WgradFew {
+  int use, rows;
+  int list[8];
+  int pad_[2];
+};
 // Weight gradient on the TMW9 tiles (fwd_tmw9.cu): the partial sums it
 // needs (floats; 0 if the plan or the input layout does not take TMW9), and
 // the launch (grad_out [n_dm][g_stride], the partials' scratch, grad_w [C]).
 int64_t tmw9_wgrad_partials(const FwdArgs& a);
-cudaError_t launch_tmw9_wgrad(const FwdArgs& a, const float* g, int64_t g_stride, float* partial, float* grad_w,
-                              cudaStream_t s);
+cudaError_t launch_tmw9_wgrad(const FwdArgs& a, const float* g, int64_t g_stride, float* partial, const WgradFew* few,
+                              float* grad_w, cudaStream_t s);
 const void* tmw9_persistent_kernel();
 const void* tmw9_plain_kernel();
 // Validated forward launch (dd_api.cpp); cfg_override < 0 uses the plan's choice.

@@ -130,6 +130,7 @@ struct WgradArgs {
   int64_t g_stride;
   float* partial;  // [C][n_part]: channel c's share from warp w of tile b at c * n_part + 12 b + w
   int64_t n_part;
+  const WgradFew* few;  // nothing to do if the gradient came from a few rows
 };
 
 // Load phases of one channel: six, each loading 16 columns of one trial
@@ -474,6 +475,7 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_tmw9_kernel(const __grid_cons
 // reduction), and wgrad_reduce_kernel adds the shares in a fixed order.
 __global__ void __launch_bounds__(kThreads, 1)
     fwd_tmw9_wgrad_kernel(const __grid_constant__ Tmw9Maps maps, FwdArgs a, WgradArgs wg) {
+  if (wg.few->use) return;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   Hdr& H = *reinterpret_cast<Hdr*>(smem_raw);
   const uint32_t sbase = smem_u32(smem_raw);
@@ -487,7 +489,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 // grad_w[c] = the sum of channel c's n_part shares: one block per channel,
 // each thread a strided subset in double, then a fixed reduction tree.
 __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* __restrict__ partial, int64_t n_part,
+                                                          const WgradFew* __restrict__ few,
                                                           float* __restrict__ grad_w) {
+  if (few->use) return;
   __shared__ double red[256];
   const int c = blockIdx.x;
   const float* row = partial + (int64_t)c * n_part;
@@ -615,8 +619,8 @@ int64_t tmw9_wgrad_partials(const FwdArgs& a) {
   return tiles * 12 * a.C;
 }
 
-cudaError_t launch_tmw9_wgrad(const FwdArgs& a, const float* g, int64_t g_stride, float* partial, float* grad_w,
-                              cudaStream_t s) {
+cudaError_t launch_tmw9_wgrad(const FwdArgs& a, const float* g, int64_t g_stride, float* partial, const WgradFew* few,
+                              float* grad_w, cudaStream_t s) {
   const int64_t n = tmw9_wgrad_partials(a);
   if (n <= 0 || g == nullptr || partial == nullptr || grad_w == nullptr) return cudaErrorInvalidConfiguration;
   Tmw9Maps maps;
@@ -627,9 +631,9 @@ cudaError_t launch_tmw9_wgrad(const FwdArgs& a, const float* g, int64_t g_stride
   dim3 grid((unsigned)((a.n_dm + kT - 1) / kT), (unsigned)((a.n_out + kBT - 1) / kBT));
   if (grid.y > 65535) return cudaErrorInvalidConfiguration;
   const int64_t n_part = n / a.C;
-  kern<<<grid, kThreads, kSmem, s>>>(maps, a, WgradArgs{g, g_stride, partial, n_part});
+  kern<<<grid, kThreads, kSmem, s>>>(maps, a, WgradArgs{g, g_stride, partial, n_part, few});
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  wgrad_reduce_kernel<<<a.C, 256, 0, s>>>(partial, n_part, grad_w);
+  wgrad_reduce_kernel<<<a.C, 256, 0, s>>>(partial, n_part, few, grad_w);
   return cudaGetLastError();
 }
 
