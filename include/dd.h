@@ -195,9 +195,10 @@ dd_status dd_check_wait_timeout(dd_plan_t plan, int64_t limit_cycles, void* stre
  *      DD_U8_I32 (DD_ERR_UNSUPPORTED otherwise).
  * out  device, [n_dm][out_row_stride] of int32 (DD_U8_I32) or float;
  *      out_row_stride >= n_out.  Overwritten; `in` and `out` must not overlap.
- * The staged kernels need `in` 16-byte aligned and in_row_stride * elem a
- * multiple of 16 bytes; inputs that are not get a plain-load kernel instead
- * (same result).  Errors: DD_ERR_ARG (null plan/in/out), DD_ERR_SHAPE (a
+ * The shared-memory kernels need `in` 16-byte aligned and take rows of any
+ * stride; the Tensor-Memory kernels need the rows that
+ * dd_plan_in_stride describes.  An input the plan's kernel cannot take gets
+ * another one that can (same result).  Errors: DD_ERR_ARG (null plan/in/out), DD_ERR_SHAPE (a
  * stride too small), DD_ERR_UNSUPPORTED, DD_ERR_CUDA (launch failure).
  */
 dd_status dd_forward(dd_plan_t plan, const void* in, int64_t in_row_stride, const float* w,

@@ -56,12 +56,11 @@ FwdArgs plan_args(const dd_plan_s* p, const void* in, int64_t in_stride, const f
 }
 
 const TileConfig* resolve_config(const dd_plan_s* p, const FwdArgs& a, int cfg_override) {
-  const int elem = p->dtype == DD_U8_I32 ? 1 : 4;
   const int k = cfg_override >= 0 ? cfg_override : p->selected;
   const TileConfig* cfg = &p->configs[k];
-  // Bulk copies need a 16-byte aligned source and row pitch; otherwise use the
-  // plain-load kernel, which computes the same sums.
-  const bool aligned = ((uintptr_t)a.in % 16 == 0) && ((a.in_stride * elem) % 16 == 0);
+  // Bulk copies start on 16-byte boundaries counted from `in`; an input that
+  // does not start on one takes the plain-load kernel, which computes the same sums.
+  const bool aligned = (uintptr_t)a.in % 16 == 0;
   auto first_of = [&](Kind kind) -> const TileConfig* {
     for (size_t j = 0; j < p->configs.size(); ++j)
       if (p->configs[j].kind == kind) return &p->configs[j];
@@ -75,6 +74,8 @@ const TileConfig* resolve_config(const dd_plan_s* p, const FwdArgs& a, int cfg_o
     cfg = t6 ? t6 : &p->configs[p->fallback];
   }
   if (cfg->kind == Kind::TmW6 && !tmw6_accepts(a.in, a.in_stride)) cfg = &p->configs[p->fallback];
+  const int elem = p->dtype == DD_U8_I32 ? 1 : 4;
+  if (a.in_stride * elem % 16 != 0 && !takes_any_rows(*cfg)) cfg = &p->configs[p->fallback];
   return cfg;
 }
 

@@ -139,6 +139,8 @@ bool tmw6_accepts(const void* in, int64_t in_stride);
 bool tmw9_accepts(const void* in, int64_t in_stride, int64_t n_in);
 int64_t tmw9_min_in_stride(int64_t n_in);
 
+// Does the configuration's kernel take rows that do not start on 16 bytes (fwd_kernels.cu)?
+bool takes_any_rows(const TileConfig& cfg);
 // Forward launch on a given configuration.
 cudaError_t launch_forward(const TileConfig& cfg, dd_dtype dtype, const FwdArgs& a, cudaStream_t s);
 
@@ -146,8 +148,8 @@ cudaError_t launch_forward(const TileConfig& cfg, dd_dtype dtype, const FwdArgs&
 // table is filled in (dd_plan.cpp).
 dd_status finish_plan(dd_plan_s* p);
 void free_plan_device(dd_plan_s* p);
-// Indices of a plan's configurations, most promising first (the measured
-// preference list, then the rest of the menu, the generic kernels last).
+// Indices of a plan's configurations, most promising first (by their time
+// estimates, then the rest of the menu).
 std::vector<int> config_preference_order(const dd_plan_s& p);
 // Forward arguments of a plan over output samples [t0, t1) (dd_api.cpp), and
 // the configuration a launch with them runs: the plan's choice (or
@@ -228,7 +230,7 @@ struct dd_plan_s {
   int64_t device_bytes = 0;
   std::vector<dd::TileConfig> configs;
   int selected = 0;
-  int fallback = 0;                   // staged configuration for inputs the selected one cannot take
+  int fallback = 0;                   // configuration for inputs the selected one cannot take
   // host-buffer forward staging (allocated on first dd_forward_host)
   void* h_dev_in = nullptr;
   void* h_dev_out = nullptr;

@@ -186,77 +186,84 @@ void free_plan_device(dd_plan_s* p) {
   p->adj_wpart_floats = 0;
 }
 
-// Default configuration: the first valid entry of a preference list, in
-// the order measured on the Table 2 setups (Apertif float: TMW9, TMW6 4.07 ms,
-// staged d8/t1024 4.94 ms; LOFAR float: staged d8/t1024 3.16 ms, d32/t384
-// 3.12 ms; Apertif uint8: U8PK 4 trials/warp c24 2.10 ms); dd_tune replaces it with a
-// measured choice.  TMW6 is offered only where a 6-trial group's offsets fit
-// its windows (Apertif, not LOFAR).
-static const char* const kPrefsF32[] = {"tmw9_f32_d9_t4096",     "tmw6_f32_d6_t4096",     "staged_d8_t1024_c4_s3",
-                                        "staged_d16_t512_c8_s3",
-                                        "staged_d32_t512_c8_s2", "staged_d32_t384_c4_s3", "staged_d16_t256_c8_s3",
-                                        "naive_t256"};
-static const char* const kPrefsU8[] = {"u8pk_w8x1_d4_c24_st3", "u8pk_w8x1_d4_c16_st3", "u8pk_w8x1_d2_c32_st3",
-                                       "u8pk_w8x1_d2_c16_st4", "staged_d16_t512_c8_s3", "staged_d8_t1024_c4_s3",
-                                       "naive_t256"};
-
-// uint8 beams with fewer than 1024 channels: two trials per warp (measured
-// on 32- and 256-channel beams of both grids: up to 2.5x faster than four)
-static const char* const kPrefsU8Narrow[] = {"u8pk_w8x1_d2_c32_st3", "u8pk_w8x1_d2_c16_st4", "u8pk_w8x1_d4_c24_st3",
-                                             "u8pk_w8x1_d4_c16_st3", "staged_d16_t512_c8_s3",
-                                             "staged_d8_t1024_c4_s3", "naive_t256"};
-
-static void pref_list(const dd_plan_s& p, const char* const** prefs, size_t* n) {
-  if (p.dtype != DD_U8_I32) {
-    *prefs = kPrefsF32;
-    *n = sizeof(kPrefsF32) / sizeof(kPrefsF32[0]);
-  } else if (p.C < 1024) {
-    *prefs = kPrefsU8Narrow;
-    *n = sizeof(kPrefsU8Narrow) / sizeof(kPrefsU8Narrow[0]);
-  } else {
-    *prefs = kPrefsU8;
-    *n = sizeof(kPrefsU8) / sizeof(kPrefsU8[0]);
+// Default configuration: the one whose time estimate is least.  The launch sizes
+// decide between the kernels (40 tiles of TMW9 leave most SMs idle, and short
+// chains of plain loads beat them), so the estimate is what was measured of
+// each on this GPU, in microseconds per channel:
+//   waves x (time of a block that shares its SM with as many as fit), but no
+//   less than the time of a block alone, plus what a launch costs.
+//                      wave   alone   measured on (channels x trials x samples)
+//   tmw9               0.303  0.303   1024 x 2048 x 20,000: 2.49 ms; x 64: 316 us
+//   staged d32 t512 c8 0.285  0.385   LOFAR beam 3.07 ms (d8 t1024 3.15); 107 x 2947 x 6576: 253 us
+//   staged d16 t512    0.156  0.27    403 x 89 x 21,373: 140 us
+//   staged d8 t1024    0.149  0.31    171 x 449 x 47,040: 478 us (d32 513)
+//   staged d8 t512     0.078  0.187   126 x 21 x 77,585: 41 us (tmw9 48)
+//   staged d8 t256     0.046  0.155   768 x 251 x 2414: 142 us (tmw9 239)
+//   u8pk 32 trials     0.165  0.257   and 3.8 us per million outputs and 256 channels (its sums leave by
+//                                     reading the output back): LOFAR 256 x 1024 x 50,000 650 us (16 trials 873)
+//   u8pk 16 trials     0.112  0.142   167 x 1618 x 27,087: 414 us (32 trials 487)
+//   u8pk 8 trials      0.075  0.104   182 x 92 x 5295: 23 us (16 trials 31)
+// A staged wave costs the more the fewer there are (the ends of blocks overlap
+// less), u8pk 1.25 times as much where long spans leave one block an SM, and 32
+// trials only pay from eight waves on (281 x 212 x 36,563: 254 us, 16 trials 165).
+// The plain kernel needs 0.030 a channel, or 2.4 T adds/s where that is more
+// (1024 x 16 x 3000: 33 us, tmw9 311, staged 158).
+static double estimate_us(const dd_plan_s& p, const TileConfig& c) {
+  constexpr double kNever = 1e30;
+  const double C = p.C, outputs = p.n_dm * (double)p.n_out;
+  const double tiles = std::ceil((double)p.n_dm / c.bd) * std::ceil((double)p.n_out / c.bt);
+  const double waves = std::ceil(tiles / 152.0);
+  auto time = [&](double wave, double alone) { return 6.0 + C * std::max(alone, waves * wave); };
+  const bool u8 = p.dtype == DD_U8_I32;
+  switch (c.kind) {
+    case Kind::Naive:
+      if (c.threads != 128) return kNever;
+      return 5.0 + std::max(0.030 * C, C * outputs / 2.4e6);
+    case Kind::TmW9:
+      return 1.0 + time(0.303, 0.303);
+    case Kind::Staged:
+      if (u8) return kNever;
+      if (c.bd == 32 && c.bt == 512 && c.cc == 8) return time(0.285 + 0.086 / waves, 0.385);
+      if (c.bd == 16 && c.bt == 512) return time(0.156 + 0.078 / waves, 0.27);
+      if (c.bd == 8 && c.bt == 1024) return time(0.149 + 0.042 / waves, 0.31);
+      if (c.bd == 8 && c.bt == 512) return time(0.078 + 0.057 / waves, 0.187);
+      if (c.bd == 8 && c.bt == 256) return time(0.046 + 0.045 / waves, 0.155);
+      return kNever;
+    case Kind::U8Pk: {
+      const double one = 2 * (c.smem + 1024) > 228 * 1024 ? 1.25 : 1.0;  // one block an SM
+      if (c.bd == 32 && c.stages == 3)
+        return waves < 8.0 ? kNever
+                           : time(0.165 * one * (c.cc == 16 ? 1.03 : 1.0), 0.257) +
+                                 3.8e-6 * outputs * std::ceil(C / 256.0);
+      if (c.bd == 16 && c.cc == 32) return time(0.112 * one, 0.142) + 0.5e-6 * outputs;
+      if (c.bd == 8 && c.threads == 128)  // two blocks an SM
+        return time(0.15 * std::ceil(waves / 2.0) / waves, 0.104) + 0.5e-6 * outputs;
+      return kNever;
+    }
+    default:
+      return kNever;
   }
 }
 
-static int preferred(const dd_plan_s& p, bool staged_only) {
-  const char* const* prefs = nullptr;
-  size_t n = 0;
-  pref_list(p, &prefs, &n);
-  for (size_t k = 0; k < n; ++k)
-    for (size_t j = 0; j < p.configs.size(); ++j)
-      if (p.configs[j].name == prefs[k] && (!staged_only || p.configs[j].kind == Kind::Staged)) return (int)j;
-  for (size_t j = 0; j < p.configs.size(); ++j)
-    if (!staged_only || p.configs[j].kind == Kind::Staged) return (int)j;
-  return 0;
-}
-static int default_config(const dd_plan_s& p) { return preferred(p, false); }
-
+// Configurations by their estimate, then the rest of the menu in its order.
 std::vector<int> config_preference_order(const dd_plan_s& p) {
-  // the preference list first (its measured order), then the rest of the
-  // menu, generic kernels last
-  const char* const* prefs = nullptr;
-  size_t n = 0;
-  pref_list(p, &prefs, &n);
-  std::vector<int> order;
-  std::vector<char> seen(p.configs.size(), 0);
-  auto take = [&](size_t j) {
-    if (!seen[j]) {
-      seen[j] = 1;
-      order.push_back((int)j);
-    }
-  };
-  for (size_t k = 0; k < n; ++k)
-    for (size_t j = 0; j < p.configs.size(); ++j)
-      if (p.configs[j].name == prefs[k] && p.configs[j].kind != Kind::Naive) take(j);
-  for (size_t j = 0; j < p.configs.size(); ++j)
-    if (p.configs[j].kind != Kind::Naive) take(j);
-  for (size_t j = 0; j < p.configs.size(); ++j) take(j);
+  std::vector<int> order(p.configs.size());
+  std::vector<double> est(p.configs.size());
+  for (size_t j = 0; j < order.size(); ++j) {
+    order[j] = (int)j;
+    est[j] = estimate_us(p, p.configs[j]);
+    // the plain kernel's other block sizes last
+    if (p.configs[j].kind == Kind::Naive && p.configs[j].threads != 128) est[j] *= 2.0;
+  }
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return est[x] < est[y]; });
   return order;
 }
-// The configuration used when the selected one cannot take an input's
-// layout (TMW6 needs 128-byte rows): the preferred shared-memory kernel.
-static int fallback_config(const dd_plan_s& p) { return preferred(p, true); }
+
+static int best_config(const dd_plan_s& p, bool any_rows) {
+  for (int j : config_preference_order(p))
+    if (!any_rows || takes_any_rows(p.configs[j])) return j;
+  return 0;
+}
 
 // Everything a plan derives from its delay table (p->delays [n_dm][C], rows
 // non-decreasing along the trial index for every channel): sizes, device
@@ -356,8 +363,10 @@ dd_status finish_plan(dd_plan_s* p) {
       p->configs.push_back(cfg);
     }
   }
-  p->selected = default_config(*p);
-  p->fallback = fallback_config(*p);
+  p->selected = best_config(*p, false);
+  // for inputs whose layout the selected one cannot take (TMW9 and TMW6 need
+  // spare samples or 128-byte rows, most others rows that start on 16 bytes)
+  p->fallback = best_config(*p, true);
   return DD_OK;
 }
 

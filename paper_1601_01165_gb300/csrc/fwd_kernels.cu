@@ -37,6 +37,12 @@ struct AccOf<uint8_t> {
 
 // ------------------------------------------------------------------ NAIVE
 
+// What bounds it on the small launches it is chosen for is the latency of one
+// load after another down the channels, so kNaiveBatch channels' delays, then
+// their samples, are all in flight before the first is added (in channel
+// order, as everywhere).
+constexpr int kNaiveBatch = 16;
+
 template <typename Tin, bool WEIGHTED>
 __global__ void __launch_bounds__(256) fwd_naive_kernel(FwdArgs a) {
   using Tacc = typename AccOf<Tin>::type;
@@ -46,9 +52,38 @@ __global__ void __launch_bounds__(256) fwd_naive_kernel(FwdArgs a) {
   if (t >= a.n_out) return;
   for (int64_t i = blockIdx.y; i < a.n_dm; i += gridDim.y) {
     const int32_t* __restrict__ drow = a.delays + i * a.C;
+    const Tin* __restrict__ col = in + t;
     Tacc acc = 0;
-    for (int c = 0; c < a.C; ++c) {
-      const Tin v = __ldg(in + (int64_t)c * a.in_stride + t + __ldg(drow + c));
+    int c = 0;
+    int32_t d[kNaiveBatch];
+    if (a.C >= kNaiveBatch) {
+#pragma unroll
+      for (int k = 0; k < kNaiveBatch; ++k) d[k] = __ldg(drow + k);
+    }
+    for (; c + kNaiveBatch <= a.C; c += kNaiveBatch) {
+      Tin v[kNaiveBatch];
+      float w[kNaiveBatch];
+      if constexpr (WEIGHTED) {
+#pragma unroll
+        for (int k = 0; k < kNaiveBatch; ++k) w[k] = __ldg(a.w + c + k);
+      }
+#pragma unroll
+      for (int k = 0; k < kNaiveBatch; ++k) v[k] = __ldg(col + (int64_t)(c + k) * a.in_stride + d[k]);
+      if (c + 2 * kNaiveBatch <= a.C) {
+#pragma unroll
+        for (int k = 0; k < kNaiveBatch; ++k) d[k] = __ldg(drow + c + kNaiveBatch + k);
+      }
+#pragma unroll
+      for (int k = 0; k < kNaiveBatch; ++k) {
+        if constexpr (WEIGHTED) {
+          acc = fmaf(w[k], v[k], acc);
+        } else {
+          acc += (Tacc)v[k];
+        }
+      }
+    }
+    for (; c < a.C; ++c) {
+      const Tin v = __ldg(col + (int64_t)c * a.in_stride + __ldg(drow + c));
       if constexpr (WEIGHTED) {
         acc = fmaf(__ldg(a.w + c), v, acc);
       } else {
@@ -135,7 +170,10 @@ __device__ __forceinline__ void stage_fetch(const FwdArgs& a, int i0, int k, int
 // All lanes of a warp: stage the warp's slots of chunk k into stage s
 // (barrier `bar`) from the delays stage_fetch read.  Each span covers samples
 // [t0 + dlo, t0 + nt + dhi) of its channel row, widened to 16-byte boundaries.
-template <typename Tin, int BD, int CC>
+// Rows need not start on one (ROWS16 false): the boundaries then count from
+// `in`, which does, and as a bulk copy may not run past the buffer, the samples
+// after its last whole 16 bytes are copied one by one.
+template <typename Tin, int BD, int CC, bool ROWS16>
 __device__ __forceinline__ void stage_issue(const FwdArgs& a, int pitch, int64_t t0, int nt, int i0, int k, int s,
                                             int slot, int lane, int32_t dlo, int32_t dhi, uint64_t* bar, Tin* sin,
                                             int32_t* sdel) {
@@ -143,19 +181,35 @@ __device__ __forceinline__ void stage_issue(const FwdArgs& a, int pitch, int64_t
   const int c = k * CC + slot;
   const bool mine = slot < CC && c < a.C;
   int64_t al = 0, ah = 0;
-  if (mine) {
-    al = (t0 + dlo) & ~(int64_t)(V - 1);
-    ah = (t0 + nt + dhi + V - 1) & ~(int64_t)(V - 1);
-    // the span fits its shared-memory row and its input row
-    if (!DD_INDEX_OK(a.status, al >= 0 && ah - al <= pitch && ah <= a.in_stride)) al = 0, ah = V;
+  if constexpr (ROWS16) {
+    if (mine) {
+      al = (t0 + dlo) & ~(int64_t)(V - 1);
+      ah = (t0 + nt + dhi + V - 1) & ~(int64_t)(V - 1);
+      // the span fits its shared-memory row and its input row
+      if (!DD_INDEX_OK(a.status, al >= 0 && ah - al <= pitch && ah <= a.in_stride)) al = 0, ah = V;
+    }
+  } else if (mine) {
+    const int64_t at = (int64_t)c * a.in_stride + t0;
+    const int64_t end = (int64_t)(a.C - 1) * a.in_stride + a.in_avail;
+    al = (at + dlo) & ~(int64_t)(V - 1);
+    ah = (at + nt + dhi + V - 1) & ~(int64_t)(V - 1);
+    if (!DD_INDEX_OK(a.status, al >= 0 && ah - al <= pitch && at + nt + dhi <= end)) al = 0, ah = V;
+    if (ah > end) {
+      ah = end & ~(int64_t)(V - 1);
+      for (int64_t e = ah; e < end; ++e)
+        sin[(size_t)(s * CC + slot) * pitch + (e - al)] = __ldg(static_cast<const Tin*>(a.in) + e);
+    }
   }
   const uint32_t bytes = mine ? (uint32_t)((ah - al) * (int64_t)sizeof(Tin)) + BD * 4 : 0u;
   const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+  if constexpr (!ROWS16) __syncwarp();  // (the samples copied one by one come before the barrier's arrival)
   if (lane == 0) mbar_arrive_expect_tx(bar, total);
   __syncwarp();
   if (mine) {
-    bulk_g2s(sin + (size_t)(s * CC + slot) * pitch, static_cast<const Tin*>(a.in) + (int64_t)c * a.in_stride + al,
-             (uint32_t)((ah - al) * (int64_t)sizeof(Tin)), bar);
+    const int64_t row = ROWS16 ? (int64_t)c * a.in_stride : 0;  // what al counts from
+    if (ROWS16 || ah > al)
+      bulk_g2s(sin + (size_t)(s * CC + slot) * pitch, static_cast<const Tin*>(a.in) + row + al,
+               (uint32_t)((ah - al) * (int64_t)sizeof(Tin)), bar);
     bulk_g2s(sdel + (s * CC + slot) * BD, a.delaysT + (int64_t)c * a.n_dm_pad + i0, BD * 4, bar);
   }
 }
@@ -163,7 +217,7 @@ __device__ __forceinline__ void stage_issue(const FwdArgs& a, int pitch, int64_t
 // A copying warp's side of the pipeline: `kn` is the next chunk it stages
 // and (dlo, dhi) its lanes' delays for it.  Every tile starts on fresh
 // barriers (a persistent block resets them between tiles).
-template <typename Tin, int BD, int CC, int STAGES, int NW, bool SPREAD>
+template <typename Tin, int BD, int CC, int STAGES, int NW, bool SPREAD, bool ROWS16>
 struct Stager {
   static_assert(STAGES >= 2, "chunk k + 1 is staged while chunk k is read");
   static_assert(CC <= (SPREAD ? 32 * NW : 32), "one lane per slot of a chunk");
@@ -194,7 +248,7 @@ struct Stager {
 #pragma unroll
     for (int j = 0; j < STAGES; ++j)
       if (j < nchunks)
-        stage_issue<Tin, BD, CC>(a, pitch, t0, nt, i0, j, j, slot(), lane, plo[j], phi[j], &B.full[j], sin, sdel);
+        stage_issue<Tin, BD, CC, ROWS16>(a, pitch, t0, nt, i0, j, j, slot(), lane, plo[j], phi[j], &B.full[j], sin, sdel);
     kn = min(STAGES, nchunks);
     stage_fetch<BD, CC>(a, i0, STAGES, slot(), dlo, dhi);
   }
@@ -214,7 +268,7 @@ struct Stager {
         if (kn > k + 1) break;  // try again at the next chunk
         if (!__any_sync(0xffffffffu, mbar_wait_bounded(&B.empty[s], par, kWaitLimitCycles))) return false;
       }
-      stage_issue<Tin, BD, CC>(a, pitch, t0, nt, i0, kn, s, slot(), lane, dlo, dhi, &B.full[s], sin, sdel);
+      stage_issue<Tin, BD, CC, ROWS16>(a, pitch, t0, nt, i0, kn, s, slot(), lane, dlo, dhi, &B.full[s], sin, sdel);
       stage_fetch<BD, CC>(a, i0, kn + 1, slot(), dlo, dhi);
       ++kn;
     }
@@ -246,7 +300,7 @@ __device__ __forceinline__ void stage_release(StageBars<STAGES>& B, int k, int l
 
 // One tile: DM trials [i0, i0 + BD) x samples [t0, t0 + BT), on fresh stage
 // barriers.  False after a timeout (also reported in the status word).
-template <typename Tin, bool WEIGHTED, int BD, int BT, int CC, int STAGES>
+template <typename Tin, bool WEIGHTED, int BD, int BT, int CC, int STAGES, bool ROWS16>
 __device__ __forceinline__ bool staged_tile(const FwdArgs& a, int pitch, int64_t t0, int i0,
                                             StageBars<STAGES>& B, unsigned char* smem_raw) {
   using Tacc = typename AccOf<Tin>::type;
@@ -257,7 +311,13 @@ __device__ __forceinline__ bool staged_tile(const FwdArgs& a, int pitch, int64_t
   static_assert(BD % NW == 0 && BT % 64 == 0 && BD % 4 == 0, "tile shape (an even number of samples per lane)");
   // a block's delay slice [i0, i0 + BD) must stay inside the padded row
   static_assert(kDmPad % BD == 0, "BD must divide the trial padding");
-  using Pipe = Stager<Tin, BD, CC, STAGES, NW, false>;
+  // Whole chunks unrolled, so that one channel's samples are on their way while
+  // the one before is added.  Full LOFAR beam, unrolled / not (ms): d32 t512 c8
+  // 3.03 / 3.12, d32 t512 c4 3.09 / 3.32, d16 t512 3.22 / 3.33; one block's 1024
+  // channels of d8 t256 0.16 / 0.18; but d8 t1024 3.58 / 3.16 and d32 t384 3.39 /
+  // 3.12, which keep the loop.
+  constexpr bool kWhole = BT != 1024 && BT != 384;
+  using Pipe = Stager<Tin, BD, CC, STAGES, NW, false, ROWS16>;
   Tin* sin = reinterpret_cast<Tin*>(smem_raw + kStBarBytes);
   int32_t* sdel = reinterpret_cast<int32_t*>(smem_raw + kStBarBytes + (size_t)STAGES * CC * pitch * sizeof(Tin));
 
@@ -287,13 +347,15 @@ __device__ __forceinline__ bool staged_tile(const FwdArgs& a, int pitch, int64_t
     const int s = k % STAGES;
     const int c0 = k * CC;
     const int cn = min(CC, a.C - c0);
-    for (int j = 0; j < cn; ++j) {
+    auto channel = [&](int j) {
       const Tin* row = sin + (size_t)(s * CC + j) * pitch;
       const int32_t* dl = sdel + (s * CC + j) * BD;
       const int d0 = dl[0];
-      const int64_t al = (t0 + d0) & ~(int64_t)(V - 1);
-      const int base = (int)(t0 + d0 - al);  // row index of (DM i0, sample t0)
-      if (!DD_INDEX_OK(a.status, base >= 0 && base + dl[BD - 1] - d0 + BT <= pitch)) continue;
+      int64_t at = t0 + d0;  // (where the row starts only matters modulo 16 bytes)
+      if constexpr (!ROWS16) at += (int64_t)(c0 + j) * a.in_stride;
+      const int64_t al = at & ~(int64_t)(V - 1);
+      const int base = (int)(at - al);  // row index of (DM i0, sample t0)
+      if (!DD_INDEX_OK(a.status, base >= 0 && base + dl[BD - 1] - d0 + BT <= pitch)) return;
       float wc = 1.0f;
       if constexpr (WEIGHTED) wc = __ldg(a.w + c0 + j);
 #pragma unroll
@@ -314,6 +376,12 @@ __device__ __forceinline__ bool staged_tile(const FwdArgs& a, int pitch, int64_t
           for (int q = 0; q < SPL; ++q) acc[m][q] += (Tacc)row[off + 32 * q];
         }
       }
+    };
+    if (kWhole && cn == CC) {
+#pragma unroll
+      for (int j = 0; j < CC; ++j) channel(j);
+    } else {
+      for (int j = 0; j < cn; ++j) channel(j);
     }
     stage_release(B, k, lane);
   }
@@ -338,11 +406,11 @@ __device__ __forceinline__ bool staged_tile(const FwdArgs& a, int pitch, int64_t
   return true;
 }
 
-template <typename Tin, bool WEIGHTED, int BD, int BT, int CC, int STAGES>
+template <typename Tin, bool WEIGHTED, int BD, int BT, int CC, int STAGES, bool ROWS16>
 __global__ void __launch_bounds__(256) fwd_staged_kernel(FwdArgs a, int pitch) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  StageBars<STAGES>& B = init_stage_bars<STAGES>(smem_raw, 8, Stager<Tin, BD, CC, STAGES, 8, false>::kCopiers);
-  (void)staged_tile<Tin, WEIGHTED, BD, BT, CC, STAGES>(a, pitch, (int64_t)blockIdx.x * BT, blockIdx.y * BD, B,
+  StageBars<STAGES>& B = init_stage_bars<STAGES>(smem_raw, 8, Stager<Tin, BD, CC, STAGES, 8, false, ROWS16>::kCopiers);
+  (void)staged_tile<Tin, WEIGHTED, BD, BT, CC, STAGES, ROWS16>(a, pitch, (int64_t)blockIdx.x * BT, blockIdx.y * BD, B,
                                                         smem_raw);
 }
 
@@ -352,7 +420,7 @@ __global__ void __launch_bounds__(256) fwd_staged_kernel(FwdArgs a, int pitch) {
 template <typename Tin, bool WEIGHTED, int BD, int BT, int CC, int STAGES>
 __global__ void __launch_bounds__(256) fwd_staged_persistent(const __grid_constant__ BatchWork w) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  constexpr int kCopiers = Stager<Tin, BD, CC, STAGES, 8, false>::kCopiers;
+  constexpr int kCopiers = Stager<Tin, BD, CC, STAGES, 8, false, true>::kCopiers;
   StageBars<STAGES>& B = init_stage_bars<STAGES>(smem_raw, 8, kCopiers);
   __shared__ int item_s;
   __shared__ BatchBeam beam_s;  // the tile's arguments, at fixed shared addresses
@@ -360,7 +428,7 @@ __global__ void __launch_bounds__(256) fwd_staged_persistent(const __grid_consta
     WorkItem it;
     if (!next_item(w, item_s, it)) break;
     copy_beam(w, it.beam, beam_s);
-    const bool ok = staged_tile<Tin, WEIGHTED, BD, BT, CC, STAGES>(beam_s.a, beam_s.pitch, (int64_t)it.x * BT,
+    const bool ok = staged_tile<Tin, WEIGHTED, BD, BT, CC, STAGES, true>(beam_s.a, beam_s.pitch, (int64_t)it.x * BT,
                                                                     it.y * BD, B, smem_raw);
     if (__syncthreads_or(!ok)) break;
     reset_stage_bars<STAGES>(B, 8, kCopiers);
@@ -392,7 +460,7 @@ struct U8PkShape {
 
 // One tile: DM trials [i0, i0 + BD) x samples [t0, t0 + BT), on fresh stage
 // barriers.  False after a timeout (also reported).
-template <int WD, int WT, int DPW, int CC, int STAGES>
+template <int WD, int WT, int DPW, int CC, int STAGES, bool ROWS16>
 __device__ __forceinline__ bool u8pk_tile(const FwdArgs& a, int pitch, int64_t t0, int i0,
                                           StageBars<STAGES>& B, unsigned char* smem_raw) {
   constexpr int V = 16;
@@ -403,7 +471,7 @@ __device__ __forceinline__ bool u8pk_tile(const FwdArgs& a, int pitch, int64_t t
   constexpr int BT = U8PkShape<WD, WT, DPW>::BT;
   static_assert(BD % 4 == 0 && BT % 16 == 0, "tile shape");
   static_assert(kDmPad % BD == 0, "BD must divide the trial padding");
-  using Pipe = Stager<uint8_t, BD, CC, STAGES, NW, true>;
+  using Pipe = Stager<uint8_t, BD, CC, STAGES, NW, true, ROWS16>;
   uint8_t* sin = smem_raw + kStBarBytes;
   int32_t* sdel = reinterpret_cast<int32_t*>(smem_raw + kStBarBytes + (size_t)STAGES * CC * pitch);
 
@@ -501,14 +569,16 @@ __device__ __forceinline__ bool u8pk_tile(const FwdArgs& a, int pitch, int64_t t
     asm("prmt.b32.f4e %0, %1, %2, %3;" : "=r"(d) : "r"(lo), "r"(hi), "r"(sel));
     return d;
   };
-  // Channel row j of stage s: the row and the offset `cj` such that trial
-  // slot i's samples for this lane start at byte cj + dl[i] of the row (the
-  // row starts at t0 + dl[0] rounded down to 16 bytes; t0 is a multiple of 16).
-  auto channel = [&](int s, int j, const uint8_t*& row, const int32_t*& dl, int& cj) {
+  // Channel row j of chunk k in stage s: the row and the offset `cj` such that
+  // trial slot i's samples for this lane start at byte cj + dl[i] of the row
+  // (the row starts at t0 + dl[0] rounded down to 16 bytes counted from `in`).
+  auto channel = [&](int k, int s, int j, const uint8_t*& row, const int32_t*& dl, int& cj) {
     row = sin + (size_t)(s * CC + j) * pitch;
     dl = sdel + (s * CC + j) * BD;
     const int d0 = dl[0];
-    cj = (int)(((uint32_t)t0 + (uint32_t)d0) & (uint32_t)(V - 1)) - d0 + lane_off;
+    uint32_t at = (uint32_t)t0 + (uint32_t)d0;
+    if constexpr (!ROWS16) at += (uint32_t)(k * CC + j) * (uint32_t)a.in_stride;
+    cj = (int)(at & (uint32_t)(V - 1)) - d0 + lane_off;
   };
   // aligned words of trial slot m of a channel row -> x[KW]
   auto aligned = [&](const uint8_t* row, const int32_t* dl, int cj, int m, uint32_t (&x)[KW]) {
@@ -544,8 +614,8 @@ __device__ __forceinline__ bool u8pk_tile(const FwdArgs& a, int pitch, int64_t t
       const uint8_t *row0, *row1;
       const int32_t *dl0, *dl1;
       int c0j, c1j;
-      channel(s, j, row0, dl0, c0j);
-      channel(s, j + 1, row1, dl1, c1j);
+      channel(k, s, j, row0, dl0, c0j);
+      channel(k, s, j + 1, row1, dl1, c1j);
 #pragma unroll
       for (int m = 0; m < DPW; ++m) {
         uint32_t x0[KW], x1[KW];
@@ -567,7 +637,7 @@ __device__ __forceinline__ bool u8pk_tile(const FwdArgs& a, int pitch, int64_t t
       const uint8_t* row0;
       const int32_t* dl0;
       int c0j;
-      channel(s, j, row0, dl0, c0j);
+      channel(k, s, j, row0, dl0, c0j);
 #pragma unroll
       for (int m = 0; m < DPW; ++m) {
         uint32_t x0[KW];
@@ -610,13 +680,13 @@ __device__ __forceinline__ bool u8pk_tile(const FwdArgs& a, int pitch, int64_t t
   return ok;
 }
 
-template <int WD, int WT, int DPW, int CC, int STAGES>
+template <int WD, int WT, int DPW, int CC, int STAGES, bool ROWS16>
 __global__ void __launch_bounds__(32 * WD * WT) fwd_u8pk_kernel(FwdArgs a, int pitch) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   using Sh = U8PkShape<WD, WT, DPW>;
   StageBars<STAGES>& B =
-      init_stage_bars<STAGES>(smem_raw, WD * WT, Stager<uint8_t, Sh::BD, CC, STAGES, WD * WT, true>::kCopiers);
-  (void)u8pk_tile<WD, WT, DPW, CC, STAGES>(a, pitch, (int64_t)blockIdx.x * Sh::BT, blockIdx.y * Sh::BD, B, smem_raw);
+      init_stage_bars<STAGES>(smem_raw, WD * WT, Stager<uint8_t, Sh::BD, CC, STAGES, WD * WT, true, ROWS16>::kCopiers);
+  (void)u8pk_tile<WD, WT, DPW, CC, STAGES, ROWS16>(a, pitch, (int64_t)blockIdx.x * Sh::BT, blockIdx.y * Sh::BD, B, smem_raw);
 }
 
 // Persistent form for batches (see fwd_staged_persistent).
@@ -624,7 +694,7 @@ template <int WD, int WT, int DPW, int CC, int STAGES>
 __global__ void __launch_bounds__(32 * WD * WT) fwd_u8pk_persistent(const __grid_constant__ BatchWork w) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   using Sh = U8PkShape<WD, WT, DPW>;
-  constexpr int kCopiers = Stager<uint8_t, Sh::BD, CC, STAGES, WD * WT, true>::kCopiers;
+  constexpr int kCopiers = Stager<uint8_t, Sh::BD, CC, STAGES, WD * WT, true, true>::kCopiers;
   StageBars<STAGES>& B = init_stage_bars<STAGES>(smem_raw, WD * WT, kCopiers);
   __shared__ int item_s;
   while (true) {
@@ -632,7 +702,7 @@ __global__ void __launch_bounds__(32 * WD * WT) fwd_u8pk_persistent(const __grid
     if (!next_item(w, item_s, it)) break;
     const BatchBeam& bm = w.beams[it.beam];  // kernel parameters
     const bool ok =
-        u8pk_tile<WD, WT, DPW, CC, STAGES>(bm.a, bm.pitch, (int64_t)it.x * Sh::BT, it.y * Sh::BD, B, smem_raw);
+        u8pk_tile<WD, WT, DPW, CC, STAGES, true>(bm.a, bm.pitch, (int64_t)it.x * Sh::BT, it.y * Sh::BD, B, smem_raw);
     if (__syncthreads_or(!ok)) break;
     reset_stage_bars<STAGES>(B, WD * WT, kCopiers);
   }
@@ -655,9 +725,31 @@ static cudaError_t launch_naive(const TileConfig& cfg, const FwdArgs& a, cudaStr
   return cudaGetLastError();
 }
 
+// Every row starts on 16 bytes: the form of a shared-memory kernel that need not
+// look where a row starts (on the Apertif uint8 beam 2.09 ms against 2.14).
+static bool rows16(const FwdArgs& a, int elem) { return a.in_stride * elem % 16 == 0; }
+// The other form exists for the shapes a plan chooses by itself (dd_plan.cpp);
+// an input whose rows do not start on 16 bytes goes to one of these.
+static constexpr bool any_rows_staged(int bd, int bt, int cc) {
+  return (bd == 8 && (bt == 256 || bt == 512)) || (bd == 16 && bt == 512) || (bd == 32 && bt == 512 && cc == 8);
+}
+static constexpr bool any_rows_u8pk(int bd, int threads, int cc) {
+  return (bd == 32 && cc != 16) || (bd == 16 && cc == 32) || (bd == 8 && threads == 128);
+}
+bool takes_any_rows(const TileConfig& cfg) {
+  if (cfg.kind == Kind::Naive) return true;
+  if (cfg.kind == Kind::Staged) return any_rows_staged(cfg.bd, cfg.bt, cfg.cc);
+  return cfg.kind == Kind::U8Pk && any_rows_u8pk(cfg.bd, cfg.threads, cfg.cc);
+}
+
 template <typename Tin, bool WEIGHTED, int BD, int BT, int CC, int STAGES>
 static cudaError_t launch_staged_t(const TileConfig& cfg, const FwdArgs& a, cudaStream_t s) {
-  auto kern = fwd_staged_kernel<Tin, WEIGHTED, BD, BT, CC, STAGES>;
+  constexpr bool kAny = any_rows_staged(BD, BT, CC);
+  auto kern = fwd_staged_kernel<Tin, WEIGHTED, BD, BT, CC, STAGES, true>;
+  if (!rows16(a, sizeof(Tin))) {
+    if (!kAny) return cudaErrorInvalidConfiguration;
+    kern = fwd_staged_kernel<Tin, WEIGHTED, BD, BT, CC, STAGES, !kAny>;
+  }
   const int smem = staged_smem_bytes<Tin>(STAGES, CC, BD, cfg.pitch);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
@@ -692,7 +784,12 @@ static cudaError_t launch_staged_t(const TileConfig& cfg, const FwdArgs& a, cuda
 
 template <int WD, int WT, int DPW, int CC, int ST>
 static cudaError_t launch_u8pk_t(const TileConfig& cfg, const FwdArgs& a, cudaStream_t s) {
-  auto kern = fwd_u8pk_kernel<WD, WT, DPW, CC, ST>;
+  constexpr bool kAny = any_rows_u8pk(WD * DPW, 32 * WD * WT, CC);
+  auto kern = fwd_u8pk_kernel<WD, WT, DPW, CC, ST, true>;
+  if (!rows16(a, 1)) {
+    if (!kAny) return cudaErrorInvalidConfiguration;
+    kern = fwd_u8pk_kernel<WD, WT, DPW, CC, ST, !kAny>;
+  }
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg.smem);
   if (e != cudaSuccess) return e;
   constexpr int BD = WD * DPW, BT = 32 * 28 * WT;
@@ -738,7 +835,6 @@ cudaError_t launch_forward(const TileConfig& cfg, dd_dtype dtype, const FwdArgs&
       return launch_tmw6(cfg, dtype, a, s);
     case Kind::TmW9:
       return launch_tmw9(cfg, dtype, a, s);
-
     case Kind::U8Pk:
       if (dtype != DD_U8_I32 || weighted) return cudaErrorInvalidConfiguration;
       return launch_u8pk(cfg, a, s);
@@ -762,9 +858,9 @@ static const void* kernel_of(const TileConfig& cfg, dd_dtype dtype, int* threads
   if (cfg.bd == BD_ && cfg.bt == BT_ && cfg.cc == CC_ && cfg.stages == ST_) {                              \
     if (dtype == DD_U8_I32)                                                                                \
       return PERSISTENT ? (const void*)fwd_staged_persistent<uint8_t, false, BD_, BT_, CC_, ST_>           \
-                        : (const void*)fwd_staged_kernel<uint8_t, false, BD_, BT_, CC_, ST_>;              \
+                        : (const void*)fwd_staged_kernel<uint8_t, false, BD_, BT_, CC_, ST_, true>;              \
     return PERSISTENT ? (const void*)fwd_staged_persistent<float, false, BD_, BT_, CC_, ST_>               \
-                      : (const void*)fwd_staged_kernel<float, false, BD_, BT_, CC_, ST_>;                  \
+                      : (const void*)fwd_staged_kernel<float, false, BD_, BT_, CC_, ST_, true>;                  \
   }
       DD_STAGED_CASES(X)
 #undef X
@@ -775,7 +871,7 @@ static const void* kernel_of(const TileConfig& cfg, dd_dtype dtype, int* threads
 #define X(WD_, WT_, DPW_, CC_, ST_)                                                                   \
   if (wd == WD_ && wt == WT_ && dpw == DPW_ && cfg.cc == CC_ && cfg.stages == ST_)                \
     return PERSISTENT ? (const void*)fwd_u8pk_persistent<WD_, WT_, DPW_, CC_, ST_>                 \
-                      : (const void*)fwd_u8pk_kernel<WD_, WT_, DPW_, CC_, ST_>;
+                      : (const void*)fwd_u8pk_kernel<WD_, WT_, DPW_, CC_, ST_, true>;
       DD_U8PK_CASES(X)
 #undef X
       return nullptr;
