@@ -196,7 +196,7 @@ dd_status dd_check_wait_timeout(dd_plan_t plan, int64_t limit_cycles, void* stre
  * out  device, [n_dm][out_row_stride] of int32 (DD_U8_I32) or float;
  *      out_row_stride >= n_out.  Overwritten; `in` and `out` must not overlap.
  * The shared-memory kernels need `in` 16-byte aligned and take rows of any
- * stride; the Tensor-Memory kernels need the rows that
+ * stride; the Tensor-Memory and grouped-sum kernels need the rows that
  * dd_plan_in_stride describes.  An input the plan's kernel cannot take gets
  * another one that can (same result).  Errors: DD_ERR_ARG (null plan/in/out), DD_ERR_SHAPE (a
  * stride too small), DD_ERR_UNSUPPORTED, DD_ERR_CUDA (launch failure).

@@ -37,6 +37,7 @@ static dd_status adjoint_plan(dd_plan_s* p, dd_plan_s** out) {
   q->n_dm = p->C;
   q->n_out = p->n_in;
   q->dtype = DD_F32_F32;
+  q->grouped = true;
   q->f_low = p->f_low;
   q->chan_bw = p->chan_bw;
   q->t_samp = p->t_samp;

@@ -26,7 +26,25 @@ struct NvtxRange {
 // 16-bit integer sums; TMW6 (float) shares each channel's input window among
 // 6 DM trials through Tensor Memory; TMW9 (float) shares it among 9 trials
 // and copies windows at 4-float granularity.
-enum class Kind : int { Naive = 0, Staged = 1, U8Pk = 4, TmW6 = 7, TmW9 = 9 };
+enum class Kind : int { Naive = 0, Staged = 1, U8Pk = 4, TmW6 = 7, TmW9 = 9, GSum = 10 };
+
+// GSUM: channels per group, and versions of a half group's sum kept in registers.
+constexpr int kGsGroup = 8;
+constexpr int kGsVersions = 6;
+constexpr int kGsChunk = 128;  // samples of a group's rows one warp makes at a time
+// A version's first offset also carries which first-half versions it joins.
+constexpr int kGsUseBit = 24;
+constexpr uint32_t kGsOffsetMask = 0xffffffu;
+// What a GSUM launch needs beside FwdArgs (device pointers; see gsum_plan.cpp).
+struct GsLaunch {
+  const uint2* idx = nullptr;   // per (trial block, channel group): first 16-byte unit, units
+  const uint4* desc = nullptr;
+  int desc_max = 0;             // bytes of the largest descriptor
+  int padp = 0;                 // staged row pitch less the tile length
+  int cap = 0;                  // row elements of one of the two buffers
+  float patterns = 0;           // patterns per block and group, on average
+  int reach = 0;                // elements from a stage's start a leaf read may touch
+};
 
 struct TileConfig {
   Kind kind;
@@ -39,6 +57,7 @@ struct TileConfig {
   int smem;     // dynamic shared memory bytes (filled per plan)
   int pitch;    // staged row pitch in elements (filled per plan)
   std::string name;
+  GsLaunch gs{};  // GSUM (filled per plan)
 };
 
 // Arguments every forward launcher receives (device pointers).
@@ -139,6 +158,23 @@ bool tmw6_accepts(const void* in, int64_t in_stride);
 bool tmw9_accepts(const void* in, int64_t in_stride, int64_t n_in);
 int64_t tmw9_min_in_stride(int64_t n_in);
 
+// Host form of a plan's GSUM descriptors for blocks of `bd` trials
+// (gsum_plan.cpp); false if the plan's delays do not fit them.
+struct GsTable {
+  int padp = 0, desc_max = 0;
+  int64_t cap = 0;                                // row elements one buffer needs
+  int64_t patterns = 0;             // over all (trial block, channel group) pairs
+  std::vector<uint2> idx;
+  std::vector<uint4> desc;
+  size_t idx_bytes() const { return idx.size() * sizeof(uint2); }
+  size_t desc_bytes() const { return desc.size() * sizeof(uint4); }
+};
+bool gsum_build(const dd_plan_s& p, int bd, int T, GsTable& t);
+// Patterns per block of `bd` trials and group, on a sample of them (-1: no descriptors).
+double gsum_patterns(const dd_plan_s& p, int bd);
+int gsum_smem_for(dd_dtype dtype, const TileConfig& cfg);
+int32_t block_spread_of(const dd_plan_s& p, int bd);
+
 // Does the configuration's kernel take rows that do not start on 16 bytes (fwd_kernels.cu)?
 bool takes_any_rows(const TileConfig& cfg);
 // Forward launch on a given configuration.
@@ -228,6 +264,8 @@ struct dd_plan_s {
   int4* d_nine_desc = nullptr;        // [ceil(n_dm / 9)][C], likewise for 9-trial groups
   int* d_status = nullptr;            // device error word
   int64_t device_bytes = 0;
+  bool grouped = false;               // float sums may add eight channels first (the adjoint's transposed plan)
+  std::vector<void*> d_gs;            // GSUM descriptors and their index
   std::vector<dd::TileConfig> configs;
   int selected = 0;
   int fallback = 0;                   // configuration for inputs the selected one cannot take

@@ -17,6 +17,7 @@ std::vector<TileConfig> staged_menu(dd_dtype dtype);
 std::vector<TileConfig> u8pk_menu(dd_dtype dtype);
 std::vector<TileConfig> tmw6_menu(dd_dtype dtype);
 std::vector<TileConfig> tmw9_menu(dd_dtype dtype);
+std::vector<TileConfig> gsum_menu(dd_dtype dtype);
 int u8pk_smem_for(const TileConfig& cfg, int pitch);
 int staged_smem_for(dd_dtype dtype, int stages, int cc, int bd, int pitch);
 
@@ -127,11 +128,60 @@ int32_t block_spread_of(const dd_plan_s& p, int bd) { return block_spread(p, bd)
 // Tensor-Memory windows (float plans).  finish_plan allocates exactly these;
 // the footprint queries report the same numbers without allocating.
 struct TableSizes {
-  size_t delays = 0, delays_t = 0, status = sizeof(int), hex = 0, nine = 0;
-  int64_t total() const { return (int64_t)(delays + delays_t + status + hex + nine); }
+  size_t delays = 0, delays_t = 0, status = sizeof(int), hex = 0, nine = 0, gsum = 0;
+  int64_t total() const { return (int64_t)(delays + delays_t + status + hex + nine + gsum); }
 };
-static TableSizes table_sizes(const dd_plan_s& p) {
+using GsumTables = std::vector<std::pair<TileConfig, GsTable>>;
+
+static double estimate_us(const dd_plan_s& p, const TileConfig& c);
+static int best_config(const dd_plan_s& p, bool any_rows);
+
+// The most patterns, by trials a block, with which sharing sums pays against the
+// other kernels of the type (Apertif grid, uint8: 13.7 of 64 trials at 1024
+// channels 1.43 ms against 2.09; about 20 at 512 the same as u8pk; float, whose
+// other kernel on a transposed plan reads shared memory once an add, further).
+// Below 192 channels nothing was gained at any size.
+static double gs_max_patterns(const dd_plan_s& p, int bd) {
+  if (p.dtype == DD_F32_F32) return 32.0;
+  if (p.C < 192) return 0.0;
+  if (bd == 64) return 18.0;
+  return p.n_dm >= 512 ? 0.0 : bd == 32 ? 14.0 : 8.0;  // small blocks are for small launches
+}
+
+// The GSUM configurations a plan gets, with their descriptors.  Float forward
+// plans get none: their kernels all add channel by channel, bit for bit the
+// same, and GSUM adds eight channels first.
+static GsumTables gsum_tables(const dd_plan_s& p) {
+  GsumTables v;
+  if (p.dtype == DD_F32_F32 && !p.grouped) return v;
+  try {
+    for (TileConfig cfg : gsum_menu(p.dtype)) {
+      const double most = gs_max_patterns(p, cfg.bd);
+      if (most <= 0.0) continue;
+      const double patterns = gsum_patterns(p, cfg.bd);
+      if (patterns < 0.0 || patterns > most) continue;
+      cfg.gs.patterns = (float)patterns;
+      // the adjoint's plan is made by the first call that needs it: only a table it will use
+      if (p.grouped && estimate_us(p, cfg) >= estimate_us(p, p.configs[best_config(p, false)])) continue;
+      GsTable t;
+      if (!gsum_build(p, cfg.bd, cfg.bt, t)) continue;
+      const int es = p.dtype == DD_U8_I32 ? 1 : 4, er = p.dtype == DD_U8_I32 ? 2 : 4;
+      cfg.gs.padp = t.padp;
+      cfg.gs.desc_max = t.desc_max;
+      cfg.gs.cap = (int)t.cap;
+      cfg.gs.reach = kGsGroup * (cfg.bt + t.padp) + cfg.cc * cfg.gs.cap * er / es;
+      cfg.smem = gsum_smem_for(p.dtype, cfg);
+      if (cfg.smem > 0) v.emplace_back(cfg, std::move(t));
+    }
+  } catch (const std::bad_alloc&) {  // the plan works without
+    v.clear();
+  }
+  return v;
+}
+
+static TableSizes table_sizes(const dd_plan_s& p, const GsumTables& gsum) {
   TableSizes t;
+  for (const auto& g : gsum) t.gsum += g.second.idx_bytes() + g.second.desc_bytes();
   const int64_t n_dm_pad = (p.n_dm + kDmPad - 1) / kDmPad * kDmPad;
   t.delays = (size_t)p.n_dm * p.C * 4;
   t.delays_t = (size_t)p.C * n_dm_pad * 4;
@@ -158,6 +208,8 @@ void free_plan_device(dd_plan_s* p) {
   cudaFree(p->d_delaysT);
   cudaFree(p->d_hex_desc);
   cudaFree(p->d_nine_desc);
+  for (void* d : p->d_gs) cudaFree(d);
+  p->d_gs.clear();
   cudaFree(p->d_status);
   cudaFree(p->h_dev_in);
   cudaFree(p->h_dev_out);
@@ -208,6 +260,10 @@ void free_plan_device(dd_plan_s* p) {
 // trials only pay from eight waves on (281 x 212 x 36,563: 254 us, 16 trials 165).
 // The plain kernel needs 0.030 a channel, or 2.4 T adds/s where that is more
 // (1024 x 16 x 3000: 33 us, tmw9 311, staged 158).
+// GSUM's times grow with the patterns its blocks have (13.7 and 8.7 on the
+// Apertif beam): 64 trials 1.43 ms there (u8pk 2.09), 32 trials 109 us on
+// 1024 x 64 x 20,000 (u8pk 145), 16 trials 76 us on 768 x 251 x 2414 (u8pk 85);
+// float, on the Apertif beam's adjoint: 3.4 ms (staged 7.1).
 static double estimate_us(const dd_plan_s& p, const TileConfig& c) {
   constexpr double kNever = 1e30;
   const double C = p.C, outputs = p.n_dm * (double)p.n_out;
@@ -240,6 +296,11 @@ static double estimate_us(const dd_plan_s& p, const TileConfig& c) {
         return time(0.15 * std::ceil(waves / 2.0) / waves, 0.104) + 0.5e-6 * outputs;
       return kNever;
     }
+    case Kind::GSum:
+      if (!u8) return time(0.12 + 0.0065 * c.gs.patterns, 0.20);
+      if (c.bd == 64) return time(0.050 + 0.0065 * c.gs.patterns, 0.128);
+      if (c.bd == 32) return time(0.060 + 0.0048 * c.gs.patterns, 0.104);
+      return time(0.060 + 0.0025 * c.gs.patterns, 0.093);
     default:
       return kNever;
   }
@@ -279,7 +340,7 @@ dd_status finish_plan(dd_plan_s* p) {
   for (int32_t c = 0; c < p->C; ++c)
     for (int32_t i = 0; i < p->n_dm_pad; ++i)
       dT[(size_t)c * p->n_dm_pad + i] = p->delays[(size_t)std::min(i, p->n_dm - 1) * p->C + c];
-  const TableSizes sizes = table_sizes(*p);
+  const TableSizes sizes = table_sizes(*p, {});
   const size_t bytes_d = sizes.delays, bytes_dT = sizes.delays_t;
   cudaError_t e = cudaMalloc(&p->d_delays, bytes_d);
   if (e == cudaSuccess) e = cudaMalloc(&p->d_delaysT, bytes_dT);
@@ -362,6 +423,25 @@ dd_status finish_plan(dd_plan_s* p) {
       if ((p->n_out + cfg.bt - 1) / cfg.bt > 65535) continue;
       p->configs.push_back(cfg);
     }
+  }
+  for (auto& [cfg, t] : gsum_tables(*p)) {
+    void* d[2] = {nullptr, nullptr};
+    const void* h[2] = {t.idx.data(), t.desc.data()};
+    const size_t n[2] = {t.idx_bytes(), t.desc_bytes()};
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+      e = cudaMalloc(&d[k], n[k]);
+      if (e == cudaSuccess) p->d_gs.push_back(d[k]);
+      if (e == cudaSuccess) e = cudaMemcpy(d[k], h[k], n[k], cudaMemcpyHostToDevice);
+    }
+    if (e != cudaSuccess) {
+      free_plan_device(p);
+      return e == cudaErrorMemoryAllocation ? set_error(DD_ERR_NOMEM, "dd_plan: device allocation failed")
+                                            : set_cuda_error("dd_plan: upload", e);
+    }
+    p->device_bytes += (int64_t)(n[0] + n[1]);
+    cfg.gs.idx = static_cast<const uint2*>(d[0]);
+    cfg.gs.desc = static_cast<const uint4*>(d[1]);
+    if ((p->n_out + cfg.bt - 1) / cfg.bt <= 65535) p->configs.push_back(cfg);
   }
   p->selected = best_config(*p, false);
   // for inputs whose layout the selected one cannot take (TMW9 and TMW6 need
@@ -495,7 +575,7 @@ extern "C" dd_status dd_plan_footprint(int32_t channels, double f_low_mhz, doubl
   dd_plan_s p;
   dd_status st = host_plan(p, channels, f_low_mhz, chan_bw_mhz, t_samp_s, dm_first, dm_step, n_dm, 1, dtype);
   if (st != DD_OK) return st;
-  *device_bytes = table_sizes(p).total();
+  *device_bytes = table_sizes(p, gsum_tables(p)).total();
   return DD_OK;
 }
 
@@ -508,7 +588,7 @@ extern "C" dd_status dd_stream_footprint(int32_t channels, double f_low_mhz, dou
   dd_plan_s p;  // the stream's own plan: the same geometry, n_out = chunk_len
   dd_status st = host_plan(p, channels, f_low_mhz, chan_bw_mhz, t_samp_s, dm_first, dm_step, n_dm, chunk_len, dtype);
   if (st != DD_OK) return st;
-  *device_bytes = table_sizes(p).total() + stream_buffer_bytes(p);
+  *device_bytes = table_sizes(p, gsum_tables(p)).total() + stream_buffer_bytes(p);
   return DD_OK;
 }
 

@@ -821,6 +821,7 @@ static cudaError_t launch_staged(const TileConfig& cfg, const FwdArgs& a, cudaSt
 
 cudaError_t launch_tmw6(const TileConfig& cfg, dd_dtype dtype, const FwdArgs& a, cudaStream_t s);
 cudaError_t launch_tmw9(const TileConfig& cfg, dd_dtype dtype, const FwdArgs& a, cudaStream_t s);
+cudaError_t launch_gsum(const TileConfig& cfg, dd_dtype dtype, const FwdArgs& a, cudaStream_t s);
 
 cudaError_t launch_forward(const TileConfig& cfg, dd_dtype dtype, const FwdArgs& a, cudaStream_t s) {
   const bool weighted = a.w != nullptr;
@@ -835,6 +836,8 @@ cudaError_t launch_forward(const TileConfig& cfg, dd_dtype dtype, const FwdArgs&
       return launch_tmw6(cfg, dtype, a, s);
     case Kind::TmW9:
       return launch_tmw9(cfg, dtype, a, s);
+    case Kind::GSum:
+      return launch_gsum(cfg, dtype, a, s);
     case Kind::U8Pk:
       if (dtype != DD_U8_I32 || weighted) return cudaErrorInvalidConfiguration;
       return launch_u8pk(cfg, a, s);
