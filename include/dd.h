@@ -268,7 +268,8 @@ dd_status dd_adjoint(dd_plan_t plan, const float* grad_out, int64_t go_row_strid
  * *result (device memory).  Rows with s_i = 0 have no S/N and are skipped;
  * valid = 0 if all are.  If grad (device, [n_rows][grad_stride]) is not NULL
  * it receives d loss / d x: nonzero only in the best row.  Sums are taken in
- * double.  Scratch: n_rows * 32 bytes from the stream-ordered allocator.
+ * double.  Scratch: with grad, its own rows while the call runs; without,
+ * n_rows * 32 bytes from the stream-ordered allocator.
  * Errors: DD_ERR_ARG, DD_ERR_SHAPE (n_cols < 8, strides), DD_ERR_NOMEM, DD_ERR_CUDA.
  */
 typedef struct {

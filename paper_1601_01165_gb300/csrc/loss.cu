@@ -21,12 +21,34 @@ namespace dd {
 
 constexpr int kBox = 8;
 
-struct RowStat {
+struct __align__(16) RowStat {
   double z;      // best S/N in the row (-inf if the row is constant)
   double mean;
   double sd;
   int64_t t;     // boxcar start of the best S/N
 };
+
+// Row i's statistics are eight words at stats + i * stride: in a scratch array,
+// or, when a gradient is asked for, in the first eight samples of its row
+// (cleared again with the gradient's own row), which needs no allocation.
+__device__ __forceinline__ void put_stat(float* at, const RowStat& r) {
+  static_assert(sizeof(RowStat) == 8 * sizeof(float), "eight words, the shortest row");
+  const int4* v = reinterpret_cast<const int4*>(&r);
+  const int w[8] = {v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w};
+#pragma unroll
+  for (int k = 0; k < 8; ++k) at[k] = __int_as_float(w[k]);
+}
+__device__ __forceinline__ RowStat get_stat(const float* at) {
+  int w[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) w[k] = __float_as_int(at[k]);
+  RowStat r;
+  r.z = __hiloint2double(w[1], w[0]);
+  r.mean = __hiloint2double(w[3], w[2]);
+  r.sd = __hiloint2double(w[5], w[4]);
+  r.t = (int64_t)((uint64_t)(uint32_t)w[7] << 32 | (uint32_t)w[6]);
+  return r;
+}
 
 __device__ __forceinline__ double boxcar(const float* row, int64_t t) {
   double b = 0.0;
@@ -148,7 +170,7 @@ __device__ __forceinline__ void boxcars(const float* x, F visit) {
 // the clearing after them, and 0.1 ms for the one row of the gradient).
 template <int NT, int K, bool ZERO>
 __global__ void __launch_bounds__(NT) snr_rows_kernel(const float* __restrict__ x, int64_t stride, int64_t n_cols,
-                                                      RowStat* __restrict__ stats, float* __restrict__ grad,
+                                                      float* stats, int64_t stats_stride, float* grad,
                                                       int64_t grad_stride) {
   constexpr int TILE = NT * K;
   __shared__ float tile[TILE + kBox - 1];
@@ -233,7 +255,7 @@ __global__ void __launch_bounds__(NT) snr_rows_kernel(const float* __restrict__ 
   const int64_t t_top = tbest[0];
   __syncthreads();
   if (!(sd > 0.0)) {
-    if (tid == 0) stats[i] = RowStat{-DBL_MAX, mean, sd, -1};
+    if (tid == 0) put_stat(stats + i * stats_stride, RowStat{-DBL_MAX, mean, sd, -1});
     return;
   }
   const double z_top = (b_top - mean) / sd;
@@ -257,20 +279,21 @@ __global__ void __launch_bounds__(NT) snr_rows_kernel(const float* __restrict__ 
     if (tid < h) tbest[tid] = min(tbest[tid], tbest[tid + h]);
     __syncthreads();
   }
-  if (tid == 0) stats[i] = RowStat{z_top, mean, sd, tbest[0]};
+  if (tid == 0) put_stat(stats + i * stats_stride, RowStat{z_top, mean, sd, tbest[0]});
 }
 
 // One block: the best row (first on ties) -> result.
 template <int NT>
-__global__ void __launch_bounds__(NT) snr_pick_kernel(const RowStat* __restrict__ stats, int n_rows,
+__global__ void __launch_bounds__(NT) snr_pick_kernel(const float* __restrict__ stats, int64_t stride, int n_rows,
                                                       dd_snr_result* __restrict__ result) {
   __shared__ double zb[NT];
   __shared__ int ib[NT];
   double z = -DBL_MAX;
   int bi = -1;
   for (int i = threadIdx.x; i < n_rows; i += NT) {
-    if (stats[i].t >= 0 && stats[i].z > z) {
-      z = stats[i].z;
+    const RowStat r = get_stat(stats + i * stride);
+    if (r.t >= 0 && r.z > z) {
+      z = r.z;
       bi = i;
     }
   }
@@ -292,11 +315,12 @@ __global__ void __launch_bounds__(NT) snr_pick_kernel(const RowStat* __restrict_
     dd_snr_result r{};
     const int b = ib[0];
     if (b >= 0) {
-      r.snr = stats[b].z;
-      r.loss = -stats[b].z;
-      r.mean = stats[b].mean;
-      r.std = stats[b].sd;
-      r.best_t = stats[b].t;
+      const RowStat best = get_stat(stats + b * stride);
+      r.snr = best.z;
+      r.loss = -best.z;
+      r.mean = best.mean;
+      r.std = best.sd;
+      r.best_t = best.t;
       r.best_row = b;
       r.valid = 1;
     } else {
@@ -313,8 +337,11 @@ __global__ void __launch_bounds__(NT) snr_pick_kernel(const RowStat* __restrict_
 // term is now made once, by multiplications, and shared through the block.
 template <int NT>
 __global__ void __launch_bounds__(NT) snr_grad_kernel(const float* __restrict__ x, int64_t stride, int64_t n_cols,
-                                                      const dd_snr_result* __restrict__ result,
+                                                      const dd_snr_result* __restrict__ result, int n_rows,
                                                       float* __restrict__ grad, int64_t grad_stride) {
+  // the other rows' statistics make place
+  for (int64_t k = (int64_t)blockIdx.x * NT + threadIdx.x; k < (int64_t)n_rows * kBox; k += (int64_t)gridDim.x * NT)
+    if (!result->valid || k / kBox != result->best_row) grad[k / kBox * grad_stride + k % kBox] = 0.0f;
   __shared__ double db[NT + kBox - 1];  // d snr / d b of the starts [u0 - 7, u0 + NT)
   if (!result->valid) return;
   const dd_snr_result r = *result;
@@ -343,14 +370,16 @@ __global__ void __launch_bounds__(NT) snr_grad_kernel(const float* __restrict__ 
 dd_status boxcar_snr_launch(const char* who, const float* x, int64_t row_stride, int32_t n_rows, int64_t n_cols,
                             dd_snr_result* result, float* grad, int64_t grad_stride, cudaStream_t s, void* scratch) {
   constexpr int NT = 256, K = 15;
-  RowStat* stats = static_cast<RowStat*>(scratch);
+  float* stats = grad ? grad : static_cast<float*>(scratch);
+  const int64_t stats_stride = grad ? grad_stride : (int64_t)(sizeof(RowStat) / sizeof(float));
   if (grad)
-    snr_rows_kernel<NT, K, true><<<n_rows, NT, 0, s>>>(x, row_stride, n_cols, stats, grad, grad_stride);
+    snr_rows_kernel<NT, K, true><<<n_rows, NT, 0, s>>>(x, row_stride, n_cols, stats, stats_stride, grad, grad_stride);
   else
-    snr_rows_kernel<NT, K, false><<<n_rows, NT, 0, s>>>(x, row_stride, n_cols, stats, nullptr, 0);
-  snr_pick_kernel<NT><<<1, NT, 0, s>>>(stats, n_rows, result);
+    snr_rows_kernel<NT, K, false><<<n_rows, NT, 0, s>>>(x, row_stride, n_cols, stats, stats_stride, nullptr, 0);
+  snr_pick_kernel<NT><<<1, NT, 0, s>>>(stats, stats_stride, n_rows, result);
   if (grad)
-    snr_grad_kernel<NT><<<(unsigned)((n_cols + NT - 1) / NT), NT, 0, s>>>(x, row_stride, n_cols, result, grad, grad_stride);
+    snr_grad_kernel<NT><<<(unsigned)((n_cols + NT - 1) / NT), NT, 0, s>>>(x, row_stride, n_cols, result, n_rows, grad,
+                                                                          grad_stride);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return set_error(DD_ERR_CUDA, "%s: launch: %s (%s)", who, cudaGetErrorString(e),
                                          cudaGetErrorName(e));
@@ -378,6 +407,10 @@ extern "C" dd_status dd_boxcar_snr(const float* x, int64_t row_stride, int32_t n
   dd_status st = boxcar_snr_check("dd_boxcar_snr", x, row_stride, n_rows, n_cols, result, grad, grad_stride);
   if (st != DD_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  // The allocator gives memory back at every synchronisation and then takes
+  // 0.2 ms to get it again, as long as the rest of the call.
+  if (grad)
+    return boxcar_snr_launch("dd_boxcar_snr", x, row_stride, n_rows, n_cols, result, grad, grad_stride, s, nullptr);
   void* scratch = nullptr;
   const size_t bytes = (size_t)n_rows * sizeof(RowStat);
   if (cudaMallocAsync(&scratch, bytes, s) != cudaSuccess)
