@@ -31,7 +31,7 @@ enum class Kind : int { Naive = 0, Staged = 1, U8Pk = 4, TmW6 = 7, TmW9 = 9, GSu
 // GSUM: channels per group, and versions of a half group's sum kept in registers.
 constexpr int kGsGroup = 8;
 constexpr int kGsVersions = 6;
-constexpr int kGsChunk = 128;  // samples of a group's rows one warp makes at a time
+constexpr int kGsChunkF32 = 128, kGsChunkU8 = 256;  // samples of a group's rows one warp makes at a time
 // A version's first offset also carries which first-half versions it joins.
 constexpr int kGsUseBit = 24;
 constexpr uint32_t kGsOffsetMask = 0xffffffu;

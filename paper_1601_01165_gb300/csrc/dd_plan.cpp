@@ -138,14 +138,14 @@ static int best_config(const dd_plan_s& p, bool any_rows);
 
 // The most patterns, by trials a block, with which sharing sums pays against the
 // other kernels of the type (Apertif grid, uint8: 13.7 of 64 trials at 1024
-// channels 1.43 ms against 2.09; about 20 at 512 the same as u8pk; float, whose
+// channels 1.39 ms against 2.09; about 20 at 512 the same as u8pk; float, whose
 // other kernel on a transposed plan reads shared memory once an add, further).
 // Below 192 channels nothing was gained at any size.
-static double gs_max_patterns(const dd_plan_s& p, int bd) {
+static double gs_max_patterns(const dd_plan_s& p, const TileConfig& c) {
   if (p.dtype == DD_F32_F32) return 32.0;
   if (p.C < 192) return 0.0;
-  if (bd == 64) return 18.0;
-  return p.n_dm >= 512 ? 0.0 : bd == 32 ? 14.0 : 8.0;  // small blocks are for small launches
+  if (p.n_dm >= 512 && (c.bd != 64 || c.bt != 576)) return 0.0;  // the other shapes are for small launches
+  return c.bd == 64 ? 18.0 : c.bd == 32 ? 14.0 : 8.0;
 }
 
 // The GSUM configurations a plan gets, with their descriptors.  Float forward
@@ -156,7 +156,7 @@ static GsumTables gsum_tables(const dd_plan_s& p) {
   if (p.dtype == DD_F32_F32 && !p.grouped) return v;
   try {
     for (TileConfig cfg : gsum_menu(p.dtype)) {
-      const double most = gs_max_patterns(p, cfg.bd);
+      const double most = gs_max_patterns(p, cfg);
       if (most <= 0.0) continue;
       const double patterns = gsum_patterns(p, cfg.bd);
       if (patterns < 0.0 || patterns > most) continue;
@@ -261,8 +261,8 @@ void free_plan_device(dd_plan_s* p) {
 // The plain kernel needs 0.030 a channel, or 2.4 T adds/s where that is more
 // (1024 x 16 x 3000: 33 us, tmw9 311, staged 158).
 // GSUM's times grow with the patterns its blocks have (13.7 and 8.7 on the
-// Apertif beam): 64 trials 1.43 ms there (u8pk 2.09), 32 trials 109 us on
-// 1024 x 64 x 20,000 (u8pk 145), 16 trials 76 us on 768 x 251 x 2414 (u8pk 85);
+// Apertif beam): 64 trials 1.39 ms there (u8pk 2.09), 32 trials 98 us on
+// 1024 x 64 x 20,000 (u8pk 145), 16 trials 75 us on 768 x 251 x 2414 (u8pk 85);
 // float, on the Apertif beam's adjoint: 3.4 ms (staged 7.1).
 static double estimate_us(const dd_plan_s& p, const TileConfig& c) {
   constexpr double kNever = 1e30;
@@ -298,9 +298,10 @@ static double estimate_us(const dd_plan_s& p, const TileConfig& c) {
     }
     case Kind::GSum:
       if (!u8) return time(0.12 + 0.0065 * c.gs.patterns, 0.20);
-      if (c.bd == 64) return time(0.050 + 0.0065 * c.gs.patterns, 0.128);
-      if (c.bd == 32) return time(0.060 + 0.0048 * c.gs.patterns, 0.104);
-      return time(0.060 + 0.0025 * c.gs.patterns, 0.093);
+      if (c.bd == 64 && c.bt == 576) return time(0.062 + 0.0078 * c.gs.patterns, 0.150);
+      if (c.bd == 64) return time(0.047 + 0.0065 * c.gs.patterns, 0.121);
+      if (c.bd == 32) return time(0.053 + 0.0047 * c.gs.patterns, 0.0);
+      return time(0.038 + 0.0035 * c.gs.patterns, 0.085);
     default:
       return kNever;
   }

@@ -21,7 +21,8 @@
 //  * One warp copies: per group of eight channels the channels' spans and the
 //    group's descriptor (gsum_plan.cpp), SS groups ahead.
 //  * NS sets of NP warps make rows, the sets taking groups in turn: a warp makes
-//    128 samples of every row of its group from the descriptor's versions.
+//    128 samples (uint8: 256) of every row of its group from the descriptor's
+//    versions.
 //  * NC warps add: one shared-memory read per trial, sample and group.
 // Rings of mbarriers join them (RB groups of rows); nothing in the group loop
 // is block-wide.
@@ -33,8 +34,9 @@
 // holds all up), row makers apart 2.5, leaves all read for every version
 // instead of the changed ones behind predicates 2.4 (a predicated-off read
 // still takes its turn), rings and two sets 1.8, three sets 1.5, spans two
-// rounds of the sets ahead (a set otherwise waits out its own copy) 1.43.
-// Eight versions kept instead of six: 1.55; rows of 576 samples: 1.63.
+// rounds of the sets ahead (a set otherwise waits out its own copy) 1.43, two
+// words a lane and tiles of 576 samples (448: 1.39 ms with four sets) 1.39.
+// Eight versions kept instead of six: 1.55; waits that suspend the warp: 1.47.
 //
 // Float sums are (x0 + x1 + x2 + x3) + (x4 + x5 + x6 + x7) within eight
 // channels, then one add to the running sum, in channel order.  8-bit sums are
@@ -125,19 +127,20 @@ struct RowMaker {
 };
 
 // ------------------------------------------------------- rows, uint8
-// Lane l makes the four samples from u = u0 + 4 l on.  A leaf is one word,
+// Lane l makes the four samples from u = u0 + 4 l on, and the four 128 further.  A leaf is one word,
 // taken from the two aligned words around it; four leaves' words added mod
 // 2^32 give A, their odd bytes in two 16-bit lanes O = S1 + 2^16 S3, and A -
 // 2^8 O = S0 + 2^16 S2.
 struct RowMakerU8 {
   static constexpr int kKeep = kGsVersions;
+  static constexpr int kWords = kGsChunkU8 / 128;  // a lane's words, 128 samples apart
   const FwdArgs& a;
   const GsLaunch& gs;
   const uint8_t* src;  // sample u of the stage (u, T and the stage are multiples of 4)
   uint16_t* dst;
   const uint16_t* end;
   int u, row_len;
-  using Sum = uint32_t[2];  // S0 + 2^16 S2, S1 + 2^16 S3
+  using Sum = uint32_t[2 * kWords];  // of each word S0 + 2^16 S2, S1 + 2^16 S3
 
   __device__ __forceinline__ RowMakerU8(const FwdArgs& a_, const GsLaunch& gs_, const uint8_t* st, uint16_t* rows,
                                         int row_len_, int u0, int lane)
@@ -145,27 +148,39 @@ struct RowMakerU8 {
         row_len(row_len_) {}
   __device__ __forceinline__ void sum(const uint4& v, Sum& t) {
     uint32_t o[4] = {v.x, v.y, v.z, v.w};
-    uint32_t A = 0u, O = 0u;
+    uint32_t A[kWords], O[kWords];
+#pragma unroll
+    for (int q = 0; q < kWords; ++q) A[q] = O[q] = 0u;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      if (!DD_INDEX_OK(a.status, (int)o[j] + u + 8 <= gs.reach)) o[j] = 0;
+      if (!DD_INDEX_OK(a.status, (int)o[j] + u + 128 * kWords - 120 <= gs.reach)) o[j] = 0;
       const uint32_t* s = reinterpret_cast<const uint32_t*>(src + (o[j] & ~3u));
-      const uint32_t x = bytes_from(s[0], s[1], o[j]);
-      A += x;
-      O += __byte_perm(x, 0u, 0x4341u);
+#pragma unroll
+      for (int q = 0; q < kWords; ++q) {
+        const uint32_t x = bytes_from(s[32 * q], s[32 * q + 1], o[j]);
+        A[q] += x;
+        O[q] += __byte_perm(x, 0u, 0x4341u);
+      }
     }
-    t[0] = A - (O << 8);
-    t[1] = O;
+#pragma unroll
+    for (int q = 0; q < kWords; ++q) {
+      t[2 * q] = A[q] - (O[q] << 8);
+      t[2 * q + 1] = O[q];
+    }
   }
   __device__ __forceinline__ void store(const Sum& x, const Sum& y) {
-    const uint32_t E = x[0] + y[0], O = x[1] + y[1];
-    if (DD_INDEX_OK(a.status, dst + 4 <= end))
-      *reinterpret_cast<uint2*>(dst) = make_uint2(__byte_perm(E, O, 0x5410u), __byte_perm(E, O, 0x7632u));
+    if (DD_INDEX_OK(a.status, dst + 128 * kWords - 124 <= end)) {
+#pragma unroll
+      for (int q = 0; q < kWords; ++q) {
+        const uint32_t E = x[2 * q] + y[2 * q], O = x[2 * q + 1] + y[2 * q + 1];
+        *reinterpret_cast<uint2*>(dst + 128 * q) = make_uint2(__byte_perm(E, O, 0x5410u), __byte_perm(E, O, 0x7632u));
+      }
+    }
     dst += row_len;
   }
 };
 
-// One warp, 128 samples of a group's rows: the versions of the first half's
+// One warp, one chunk of samples of a group's rows: the versions of the first half's
 // sum stay in registers, kKeep at a time; each version of the second
 // half's sum is made once per such batch and added to those it occurs with.
 template <typename Maker>
@@ -401,6 +416,7 @@ __global__ void __launch_bounds__(32 * (NC + NS * NP + 1), MB) fwd_gsum_kernel(F
   }
 
   if (warp >= NC) {
+    constexpr int kChunk = sizeof(Tin) == 1 ? kGsChunkU8 : kGsChunkF32;
     const int set = (warp - NC) / NP, pw = (warp - NC) % NP;
     for (int g = set; g < ng; g += NS) {
       const int k = g % SS, r = g % RB;
@@ -411,7 +427,7 @@ __global__ void __launch_bounds__(32 * (NC + NS * NP + 1), MB) fwd_gsum_kernel(F
         const uint4 h = d[0];
         if (pw == NP - 1)
           for (int m = lane; m < BD; m += 32) offs[r * BD + m] = reinterpret_cast<const uint32_t*>(d + 1)[m];
-        for (int u0 = 128 * pw; u0 < (int)h.y; u0 += 128 * NP) {
+        for (int u0 = kChunk * pw; u0 < (int)h.y; u0 += kChunk * NP) {
           typename GsTypes<Tin>::Maker mk(a, gs, reinterpret_cast<const Tin*>(sring + k * stage_bytes),
                                           rows + r * gs.cap, (int)h.y, u0, lane);
           make_rows(mk, d + 1 + BD / 4, (int)h.x);
@@ -472,9 +488,10 @@ __global__ void __launch_bounds__(32 * (NC + NS * NP + 1), MB) fwd_gsum_kernel(F
 #define DD_GSUM_F32(X)                 \
   X(float, 16, 2, 5, 4, 12, 2, 2, 1)
 #define DD_GSUM_U8(X)                  \
-  X(uint8_t, 16, 3, 5, 4, 14, 6, 4, 1) \
-  X(uint8_t, 8, 2, 5, 4, 14, 4, 3, 1)  \
-  X(uint8_t, 8, 2, 4, 2, 14, 4, 3, 2)
+  X(uint8_t, 16, 3, 3, 4, 18, 6, 3, 1) \
+  X(uint8_t, 16, 4, 3, 4, 14, 4, 4, 1) \
+  X(uint8_t, 8, 3, 3, 4, 14, 6, 4, 1)  \
+  X(uint8_t, 8, 2, 2, 2, 14, 4, 3, 2)
 
 #define GS_P NC, NS, NP, DPW, SPL, SS, RB, MB
 template <typename Tin, int NC, int NS, int NP, int DPW, int SPL, int SS, int RB, int MB>

@@ -89,7 +89,8 @@ static void build_blocks(const dd_plan_s& p, int bd, int T, int padp, int b0, in
         if (s == 0 || rank(k) != rank(by[s - 1])) order[n_p++] = k;
       }
       // every row covers the shifts of the whole block, in whole chunks
-      const int row_len = (T + e[bd - 1] + kGsChunk - 1) / kGsChunk * kGsChunk;
+      const int chunk = es == 1 ? kGsChunkU8 : kGsChunkF32;
+      const int row_len = (T + e[bd - 1] + chunk - 1) / chunk * chunk;
       t.cap = std::max<int64_t>(t.cap, (int64_t)n_p * row_len);
       t.patterns += n_p;
       const size_t at = t.desc.size();

@@ -20,7 +20,7 @@ def _gsum(plan):
 
 @pytest.mark.parametrize("C,n_dm,n_out,dm0", [
     (193, 1, 1, 0.0), (199, 15, 447, 0.0), (200, 17, 448, 0.0), (250, 33, 449, 300.0), (257, 64, 1345, 0.0),
-    (515, 65, 900, 40.0), (1024, 31, 1931, 400.0), (1022, 130, 463, 0.0),
+    (515, 65, 900, 40.0), (1024, 31, 1931, 400.0), (1022, 130, 463, 0.0), (1024, 70, 577, 0.0), (777, 64, 1151, 200.0),
 ])
 @pytest.mark.parametrize("saturated", [False, True], ids=["noise", "saturated"])
 def test_u8_every_shape_is_exact(C, n_dm, n_out, dm0, saturated):
