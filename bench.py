@@ -72,7 +72,7 @@ def _kernel_hash():
     import re
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1601_01165_gb300", "csrc")
-    for name in ("fwd_kernels.cu", "fwd_tmw6.cu", "fwd_tmw9.cu", "ptx.cuh", "dd_internal.h"):
+    for name in ("fwd_kernels.cu", "fwd_gsum.cu", "fwd_tmw6.cu", "fwd_tmw9.cu", "ptx.cuh", "dd_internal.h"):
         with open(os.path.join(csrc, name)) as f:
             text = f.read()
         text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)

@@ -283,7 +283,8 @@ static double estimate_us(const dd_plan_s& p, const TileConfig& c) {
       if (c.bd == 16 && c.bt == 512) return time(0.156 + 0.078 / waves, 0.27);
       if (c.bd == 8 && c.bt == 1024) return time(0.149 + 0.042 / waves, 0.31);
       if (c.bd == 8 && c.bt == 512) return time(0.078 + 0.057 / waves, 0.187);
-      if (c.bd == 8 && c.bt == 256) return time(0.046 + 0.045 / waves, 0.155);
+      if (c.bd == 8 && c.bt == 256)  // long spans cost its short tiles most (293 x 1081 x 1064, LOFAR: 0.067)
+        return time((0.046 + 0.045 / waves) * (1.0 + 0.22 * (c.pitch - c.bt) / c.bt), 0.155);
       return kNever;
     case Kind::U8Pk: {
       const double one = 2 * (c.smem + 1024) > 228 * 1024 ? 1.25 : 1.0;  // one block an SM
