@@ -49,10 +49,10 @@ SM_MAX_MHZ_NOMINAL = 2070.0
 # keyed by (setup name, output samples, kernel config, dtype); valid only while
 # the kernel source hash matches.
 NCU_TRAFFIC = {
-    # fwd_tmw9_kernel<0>: 111.1 MB read + 123.0 MB written
-    ("apertif", 20000, "tmw9_f32_d9_t4096", "f32"): {"bytes": 234_030_848, "hash": "e4f86a4a09fcbaf3"},
-    # fwd_u8pk_kernel<8,1,4,24,3>: 32.7 MB read + 111.9 MB written
-    ("apertif", 20000, "u8pk_w8x1_d4_c24_st3", "u8"): {"bytes": 144_604_928, "hash": "e4f86a4a09fcbaf3"},
+    # fwd_tmw9_kernel<0>: 110.8 MB read + 123.1 MB written
+    ("apertif", 20000, "tmw9_f32_d9_t4096", "f32"): {"bytes": 233_860_608, "hash": "28f26e0e6f2662ad"},
+    # fwd_gsum_kernel<uint8, 16, 3, 3, 4, 18, 6, 3, 1>: 39.5 MB read + 114.2 MB written
+    ("apertif", 20000, "gsum8_w16p3x3_d4_s18_r63", "u8"): {"bytes": 153_761_792, "hash": "28f26e0e6f2662ad"},
 }
 
 

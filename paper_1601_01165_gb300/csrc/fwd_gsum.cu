@@ -27,7 +27,7 @@
 // Rings of mbarriers join them (RB groups of rows); nothing in the group loop
 // is block-wide.
 //
-// What bounds it is shared memory (57-70 % of its cycles on float) and the
+// What bounds it is shared memory (57 % of its cycles on uint8, 70 on float) and the
 // chain of its reads in the row makers.  One Apertif uint8 beam (1024 x 2048 x
 // 20,000; u8pk takes 2.09 ms), each step measured: every warp making rows and
 // adding between two block barriers 3.7 ms (one warp's chain of dependent reads
