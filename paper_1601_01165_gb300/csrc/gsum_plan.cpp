@@ -7,29 +7,20 @@
 // rel_k[j] = (d[k][j] - d[0][j]) - e_k; trials with equal patterns read one
 // row at their own shifts.  Row sample u of pattern p adds leaf j at staged
 // sample  (d[0][j] mod V) + rel_p[j] + u  of its span (which starts at d[0][j]
-// rounded down to V samples, 16 bytes).  A row covers u from its smallest
-// shift (rounded down to A) to its largest (rounded up to A) plus the tile's
-// T samples; T is the kernel's, so the descriptor keeps both parts of an
-// address apart: multiples of T and the rest.
+// rounded down to V samples, 16 bytes).  Every row of a (block, group) covers u
+// in [0, T + e of the last trial), rounded up to whole chunks of a row maker.
 //
 // The sum of a group is the sum of its two halves' (leaves 0-3 and 4-7), and
 // a half has few versions (relative delays of its own four leaves) in a block.
 // One descriptor, in 16-byte units:
-//   [0]            x = batches, y = the block's largest shift e, z = first
-//                  unit of the rows' records
-//   [1 .. BD/4]    per trial: row number << 16 | rest of the row address of
-//                  its first sample
+//   [0]            x = batches, y = row length, z = rows
+//   [1 .. BD/4]    per trial: where its first sample is, in row elements
 //   then per batch of up to kGsVersions versions of the first half:
 //     x = versions of the first half in it, y = of the second half that occur
 //     with them; then those versions' units, the first half's first
-//   A version: x, y = the leaves' staged positions at u = 0 (16 bits each),
-//     less leaf number times T; z = which leaves differ from the version
-//     before (all in a batch's first); w (second half) = with which of the
-//     batch's first-half versions it makes a row
-//   then the rows' records in the order made, two to a unit:
-//     rest of the address of the row's sample u = 0 (signed, 16 bits) | first
-//     u << 16, last shift | row number << 16
-// Versions are sorted, so most differ from the one before in one leaf.
+//   A version: the staged byte offsets of its four leaves at u = 0; a second
+//     half's first offset carries, from bit kGsUseBit, with which of the
+//     batch's first-half versions it makes a row (rows are in that order)
 #include <algorithm>
 #include <cstring>
 #include <future>
