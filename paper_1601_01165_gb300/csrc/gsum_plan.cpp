@@ -143,7 +143,8 @@ double gsum_patterns(const dd_plan_s& p, int bd) {
   const int pad = pitch_pad(p, bd);
   if (pad < 0) return -1.0;
   GsTable t;
-  const int n_b = (p.n_dm + bd - 1) / bd, n_g = (p.C + kGsGroup - 1) / kGsGroup;
+  // (whole blocks: a last one of few trials has few patterns but takes as long)
+  const int n_b = std::max(1, p.n_dm / bd), n_g = (p.C + kGsGroup - 1) / kGsGroup;
   for (int k = 0; k < 4; ++k) {
     const int b = (int)((int64_t)k * n_b / 4);
     build_blocks(p, bd, 512, pad, b, b + 1, std::max(1, n_g / 16), t);
