@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(256) wgrad_scan_kernel(const float* __restrict
   if (threadIdx.x == 0) any[blockIdx.x] = found;
 }
 
-// One block: few.rows, few.list (ascending) and few.use.
+// One block: few.rows, few.list (ascending), few.use, and few.bad cleared.
 __global__ void __launch_bounds__(1024) wgrad_list_kernel(const int* __restrict__ any, int n_rows, WgradFew* few) {
   __shared__ int cnt[1024];
   const int per = (n_rows + 1023) / 1024, i0 = (int)threadIdx.x * per, i1 = min(n_rows, i0 + per);
@@ -146,17 +146,19 @@ __global__ void __launch_bounds__(1024) wgrad_list_kernel(const int* __restrict_
   if (threadIdx.x == 0) {
     few->rows = total;
     few->use = use ? 1 : 0;
+    few->bad = 0;
   }
 }
 
-// few.use = 0 if a sample of the input is not finite.
+// few.bad if a sample of the input is not finite.  (The block's threads all
+// return or all reach the barrier: this kernel does not write few.use.)
 __global__ void __launch_bounds__(256) wgrad_finite_kernel(const float* __restrict__ in, int64_t stride, int64_t n,
                                                            WgradFew* few) {
   if (!few->use) return;
   const float* row = in + (int64_t)blockIdx.x * stride;
   bool bad = false;
   for (int64_t t = threadIdx.x; t < n; t += 256) bad |= !(fabsf(__ldg(row + t)) <= 3.402823466e38f);
-  if (__syncthreads_or(bad) && threadIdx.x == 0) few->use = 0;
+  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicExch(&few->bad, 1);
 }
 
 // grad_w[c] of the listed rows, one block per channel: four short float chains
@@ -165,7 +167,7 @@ __global__ void __launch_bounds__(256) wgrad_rows_kernel(const float* __restrict
                                                          const float* __restrict__ in, int64_t in_stride,
                                                          const int32_t* __restrict__ delays, int C, int64_t n,
                                                          const WgradFew* __restrict__ few, float* __restrict__ grad_w) {
-  if (!few->use) return;
+  if (!few->done()) return;
   const int c = blockIdx.x, rows = few->rows;
   double sum = 0.0;
   for (int r = 0; r < rows; ++r) {

@@ -207,12 +207,17 @@ cudaError_t launch_persistent(const TileConfig& cfg, dd_dtype dtype, const Batch
                               cudaStream_t s);
 size_t tmw9_views_bytes();
 bool tmw9_encode_views(const FwdArgs& a, void* out);
-// The rows of grad_out that have a nonzero, if few (adjoint.cu): with `use`
-// the weight gradient has been computed from them and the tiles do nothing.
+// The rows of grad_out that have a nonzero, if few (adjoint.cu): with `use`,
+// unless `bad`, the weight gradient has been computed from them and the tiles
+// do nothing.  `bad` has a word of its own: the kernel that looks for samples
+// that are not finite runs only with `use`, and all its threads have to agree.
 struct WgradFew {
-  int use, rows;
+  int use, bad, rows;
   int list[8];
-  int pad_[2];
+  int pad_[1];
+#ifdef __CUDACC__
+  __device__ __forceinline__ bool done() const { return use && !bad; }
+#endif
 };
 // Weight gradient on the TMW9 tiles (fwd_tmw9.cu): the partial sums it
 // needs (floats; 0 if the plan or the input layout does not take TMW9), and

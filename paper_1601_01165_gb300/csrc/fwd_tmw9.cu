@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_tmw9_kernel(const __grid_cons
 // reduction), and wgrad_reduce_kernel adds the shares in a fixed order.
 __global__ void __launch_bounds__(kThreads, 1)
     fwd_tmw9_wgrad_kernel(const __grid_constant__ Tmw9Maps maps, FwdArgs a, WgradArgs wg) {
-  if (wg.few->use) return;
+  if (wg.few->done()) return;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   Hdr& H = *reinterpret_cast<Hdr*>(smem_raw);
   const uint32_t sbase = smem_u32(smem_raw);
@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* __restrict__ partial, int64_t n_part,
                                                           const WgradFew* __restrict__ few,
                                                           float* __restrict__ grad_w) {
-  if (few->use) return;
+  if (few->done()) return;
   __shared__ double red[256];
   const int c = blockIdx.x;
   const float* row = partial + (int64_t)c * n_part;
