@@ -21,6 +21,7 @@
 
 #include "dd_internal.h"
 #include "ptx.cuh"
+#include "spans.h"
 
 namespace dd {
 
@@ -171,8 +172,9 @@ __device__ __forceinline__ void stage_fetch(const FwdArgs& a, int i0, int k, int
 // (barrier `bar`) from the delays stage_fetch read.  Each span covers samples
 // [t0 + dlo, t0 + nt + dhi) of its channel row, widened to 16-byte boundaries.
 // Rows need not start on one (ROWS16 false): the boundaries then count from
-// `in`, which does, and as a bulk copy may not run past the buffer, the samples
-// after its last whole 16 bytes are copied one by one.
+// `in`, which does, and as a copy may not run past the last sample of the last
+// row (the rows may be a part of wider ones), the samples after its last whole
+// 16 bytes are copied one by one.
 template <typename Tin, int BD, int CC, bool ROWS16>
 __device__ __forceinline__ void stage_issue(const FwdArgs& a, int pitch, int64_t t0, int nt, int i0, int k, int s,
                                             int slot, int lane, int32_t dlo, int32_t dhi, uint64_t* bar, Tin* sin,
@@ -190,15 +192,14 @@ __device__ __forceinline__ void stage_issue(const FwdArgs& a, int pitch, int64_t
     }
   } else if (mine) {
     const int64_t at = (int64_t)c * a.in_stride + t0;
-    const int64_t end = (int64_t)(a.C - 1) * a.in_stride + a.in_avail;
-    al = (at + dlo) & ~(int64_t)(V - 1);
-    ah = (at + nt + dhi + V - 1) & ~(int64_t)(V - 1);
-    if (!DD_INDEX_OK(a.status, al >= 0 && ah - al <= pitch && at + nt + dhi <= end)) al = 0, ah = V;
-    if (ah > end) {
-      ah = end & ~(int64_t)(V - 1);
-      for (int64_t e = ah; e < end; ++e)
-        sin[(size_t)(s * CC + slot) * pitch + (e - al)] = __ldg(static_cast<const Tin*>(a.in) + e);
-    }
+    const int64_t end = input_end(a.C, a.in_stride, a.n_in);
+    RowSpan r = row_span<V>(at + dlo, at + nt + dhi, end);
+    if (!DD_INDEX_OK(a.status, r.first >= 0 && r.last - r.first <= pitch && at + nt + dhi <= end))
+      r = RowSpan{0, V, V};
+    al = r.first;
+    ah = r.bulk_end;
+    for (int64_t e = r.bulk_end; e < r.last; ++e)
+      sin[(size_t)(s * CC + slot) * pitch + (e - al)] = __ldg(static_cast<const Tin*>(a.in) + e);
   }
   const uint32_t bytes = mine ? (uint32_t)((ah - al) * (int64_t)sizeof(Tin)) + BD * 4 : 0u;
   const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
