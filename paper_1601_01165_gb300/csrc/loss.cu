@@ -102,9 +102,11 @@ __device__ __forceinline__ DF df_add(DF a, DF b) {
   return fast_two_sum(u.h, __fadd_rn(u.l, t.l));
 }
 
-// The same for the sums below, where a.l + b.l needs no exact error: two
+// The same for the boxcars, where a.l + b.l needs no exact error: two
 // operations instead of nine.  The result is within 2^-47 (|a| + |b|), and
-// exact wherever |a.l + b.l| fits 24 bits of the operands' common unit.
+// exact wherever |a.l + b.l| fits 24 bits of the operands' common unit.  (A
+// boxcar takes two of these, where one sample added after another rounds the
+// low parts six times.)
 __device__ __forceinline__ DF df_add_fast(DF a, DF b) {
   const DF s = two_sum(a.h, b.h);
   return fast_two_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
@@ -165,7 +167,7 @@ __device__ __forceinline__ void boxcars(const float* x, F visit) {
 // with that S/N lies among those whose boxcar is within rounding of b_max:
 // only a thread that has another boxcar that close goes over its starts again
 // (a different start only when two sums round to one S/N).
-// 2048 x 20,000 with the gradient: the whole call 204 us, nearly all of it this
+// 2048 x 20,000 with the gradient: the whole call 224 us, nearly all of it this
 // kernel (before: 493, every boxcar summed by itself in each of three passes,
 // the clearing after them, and 0.1 ms for the one row of the gradient).
 template <int NT, int K, bool ZERO>
@@ -219,9 +221,9 @@ __global__ void __launch_bounds__(NT) snr_rows_kernel(const float* __restrict__ 
     const int n = (int)max((int64_t)0, min((int64_t)K, nb - t0));
     auto visit = [&](int k, DF b) {
       if (k < n) {
-        const DF c = two_sum(b.h, neg_mean.h);
-        const DF d = fast_two_sum(c.h, __fadd_rn(c.l, __fadd_rn(b.l, neg_mean.l)));
-        v = df_add_fast(v, df_sqr(d));
+        // (the whole sums: where b is close to a large mean, nothing but the
+        // low parts' exact sum is left of the difference)
+        v = df_add(v, df_sqr(df_add(b, neg_mean)));
         if (at < 0 || df_gt(b, bmax)) {  // t increases, so the first maximum is kept
           before = bmax;
           bmax = b;
