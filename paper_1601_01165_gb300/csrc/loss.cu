@@ -183,22 +183,28 @@ __global__ void __launch_bounds__(NT) snr_rows_kernel(const float* __restrict__ 
   const int64_t nb = n_cols - kBox + 1;
 
   // pass 1: the sum of the boxcars (a sample u is in min(u + 1, 8, n_cols - u, nb) of them)
-  DF s4[4] = {};
-  int64_t u = tid;
-  for (; u + 3 * NT < n_cols; u += 4 * NT) {
-    float v[4];
+  double sum = 0.0;
+  if (nb < kBox) {
+    // Few starts share most of their samples, and may differ by less than the
+    // boxcars' own rounding: their mean is that of the boxcars as pass 2 has
+    // them (one start has no deviation, two have S/N 1).
+    if (tid < nb) boxcars<1>(row + tid, [&](int, DF b) { sum = df_value(b); });
+  } else {
+    DF s4[4] = {};
+    int64_t u = tid;
+    for (; u + 3 * NT < n_cols; u += 4 * NT) {
+      float v[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = __ldg(row + u + k * NT);
+      for (int k = 0; k < 4; ++k) v[k] = __ldg(row + u + k * NT);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) s4[k] = df_add_f(s4[k], v[k]);
-  }
-  for (; u < n_cols; u += NT) s4[0] = df_add_f(s4[0], __ldg(row + u));
-  double sum = (double)kBox * df_value(df_add(df_add(s4[0], s4[1]), df_add(s4[2], s4[3])));
-  for (int64_t e = tid; e < 2 * (kBox - 1); e += NT) {  // the ends: count the missing ones off
-    const int64_t at = e < kBox - 1 ? e : n_cols - 1 - (e - (kBox - 1));
-    const int64_t lo = min(at + 1, (int64_t)kBox), hi = min(n_cols - at, nb);
-    // (a short row's two ends may meet: each sample once)
-    if (at >= 0 && (e < kBox - 1 ? at < n_cols : at >= kBox - 1)) sum -= (double)(kBox - min(lo, hi)) * (double)__ldg(row + at);
+      for (int k = 0; k < 4; ++k) s4[k] = df_add_f(s4[k], v[k]);
+    }
+    for (; u < n_cols; u += NT) s4[0] = df_add_f(s4[0], __ldg(row + u));
+    sum = (double)kBox * df_value(df_add(df_add(s4[0], s4[1]), df_add(s4[2], s4[3])));
+    for (int64_t e = tid; e < 2 * (kBox - 1); e += NT) {  // the ends: count the missing ones off
+      const int64_t at = e < kBox - 1 ? e : n_cols - 1 - (e - (kBox - 1));
+      sum -= (double)(kBox - min(min(at + 1, n_cols - at), (int64_t)kBox)) * (double)__ldg(row + at);
+    }
   }
   const double mean = block_sum<NT>(sum, red) / (double)nb;
 
