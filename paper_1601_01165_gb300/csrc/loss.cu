@@ -167,7 +167,7 @@ __device__ __forceinline__ void boxcars(const float* x, F visit) {
 // with that S/N lies among those whose boxcar is within rounding of b_max:
 // only a thread that has another boxcar that close goes over its starts again
 // (a different start only when two sums round to one S/N).
-// 2048 x 20,000 with the gradient: the whole call 224 us, nearly all of it this
+// 2048 x 20,000 with the gradient: the whole call 226 us, nearly all of it this
 // kernel (before: 493, every boxcar summed by itself in each of three passes,
 // the clearing after them, and 0.1 ms for the one row of the gradient).
 template <int NT, int K, bool ZERO>
@@ -340,9 +340,9 @@ __global__ void __launch_bounds__(NT) snr_pick_kernel(const float* __restrict__ 
   }
 }
 
-// d loss / d x for the best row (the rows kernel cleared all).  Double divisions
-// and each boxcar eight times over made this one row cost 0.1 ms; every start's
-// term is now made once, by multiplications, and shared through the block.
+// d loss / d x for the best row (the rows kernel cleared all).  Each boxcar and
+// its double divisions eight times over made this one row cost 0.1 ms; every
+// start's term is made once, with two divisions, and shared through the block.
 template <int NT>
 __global__ void __launch_bounds__(NT) snr_grad_kernel(const float* __restrict__ x, int64_t stride, int64_t n_cols,
                                                       const dd_snr_result* __restrict__ result, int n_rows,
@@ -356,13 +356,16 @@ __global__ void __launch_bounds__(NT) snr_grad_kernel(const float* __restrict__ 
   const int64_t u0 = (int64_t)blockIdx.x * NT;
   const float* row = x + (int64_t)r.best_row * stride;
   const int64_t nb = n_cols - kBox + 1;
-  const double inv_sd = 1.0 / r.std, inv_nb = 1.0 / (double)nb;
+  // d snr / d b[t] = ((t == best) - 1/nb) / sd - snr z[t] / (nb sd); divided, not
+  // multiplied by reciprocals, so that two terms which cancel do so exactly
+  const double inv_nb = 1.0 / (double)nb, nb_sd = (double)nb * r.std;
+  const double at_best = (1.0 - inv_nb) / r.std, elsewhere = (0.0 - inv_nb) / r.std;
   for (int k = threadIdx.x; k < NT + kBox - 1; k += NT) {
     const int64_t t = u0 - (kBox - 1) + k;
     double v = 0.0;
     if (t >= 0 && t < nb) {
-      const double z = (boxcar(row, t) - r.mean) * inv_sd;
-      v = ((t == r.best_t ? 1.0 : 0.0) - inv_nb * (1.0 + r.snr * z)) * inv_sd;
+      const double z = (boxcar(row, t) - r.mean) / r.std;
+      v = (t == r.best_t ? at_best : elsewhere) - r.snr * z / nb_sd;
     }
     db[k] = v;
   }
