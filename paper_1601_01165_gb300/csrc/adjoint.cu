@@ -161,8 +161,11 @@ __global__ void __launch_bounds__(256) wgrad_finite_kernel(const float* __restri
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicExch(&few->bad, 1);
 }
 
-// grad_w[c] of the listed rows, one block per channel: four short float chains
-// a thread and row, then double; a fixed order.
+// grad_w[c] of the listed rows, one block per channel: four float chains a
+// thread, of kChain products each however long the row (the tiles end theirs
+// after 32), then double; a fixed order.
+constexpr int kChain = 16;
+
 __global__ void __launch_bounds__(256) wgrad_rows_kernel(const float* __restrict__ g, int64_t g_stride,
                                                          const float* __restrict__ in, int64_t in_stride,
                                                          const int32_t* __restrict__ delays, int C, int64_t n,
@@ -174,13 +177,17 @@ __global__ void __launch_bounds__(256) wgrad_rows_kernel(const float* __restrict
     const int i = few->list[r];
     const float* a = g + (int64_t)i * g_stride;
     const float* b = in + (int64_t)c * in_stride + delays[(int64_t)i * C + c];
-    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     int64_t t = threadIdx.x;
-    for (; t + 768 < n; t += 1024)
+    while (t < n) {
+      float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      int m = 0;
+      for (; m < kChain && t + 768 < n; ++m, t += 1024)
 #pragma unroll
-      for (int k = 0; k < 4; ++k) s[k] = fmaf(__ldg(a + t + 256 * k), __ldg(b + t + 256 * k), s[k]);
-    for (; t < n; t += 256) s[0] = fmaf(__ldg(a + t), __ldg(b + t), s[0]);
-    sum += ((double)s[0] + (double)s[1]) + ((double)s[2] + (double)s[3]);
+        for (int k = 0; k < 4; ++k) s[k] = fmaf(__ldg(a + t + 256 * k), __ldg(b + t + 256 * k), s[k]);
+      if (m < kChain)  // (the last ones, at most three)
+        for (; t < n; t += 256) s[0] = fmaf(__ldg(a + t), __ldg(b + t), s[0]);
+      sum += ((double)s[0] + (double)s[1]) + ((double)s[2] + (double)s[3]);
+    }
   }
   __shared__ double red[256];
   red[threadIdx.x] = sum;
