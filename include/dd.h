@@ -384,7 +384,10 @@ dd_status dd_batch_destroy(dd_batch_t batch);
  * dd_forward on the concatenated input.
  * chunk  device [channels][chunk_len] (element type of the plan), contiguous.
  * out    device [n_dm][chunk_len] of the plan's output type, contiguous.
- * The plan's n_out is not used by streaming; the output length is chunk_len.
+ * The plan's n_out is not used by streaming; the output length is chunk_len.  A
+ * configuration selected, tuned or taken from a tuning database for the plan is
+ * the stream's too (where its chunks allow it); otherwise the stream's own is
+ * chosen for chunk_len.
  * dd_stream_save / dd_stream_restore copy the state (tail + sample counter)
  * to / from a host buffer of dd_stream_state_bytes bytes, for checkpointing.
  * dd_stream_reset zeroes the tail on `stream` (asynchronously, ordered after

@@ -451,7 +451,10 @@ extern "C" dd_status dd_batch_tune(dd_batch_t b, double budget_s, const char* db
       if (kv.first == key) name = &kv.second;
     if (name) {
       for (size_t j = 0; j < p->configs.size(); ++j)
-        if (p->configs[j].name == *name) p->selected = (int)j;
+        if (p->configs[j].name == *name) {
+          p->selected = (int)j;
+          p->chosen_by = ChosenBy::Caller;
+        }
       continue;
     }
     st = dd_tune(p, budget_s, db_path, nullptr);

@@ -46,6 +46,12 @@ struct GsLaunch {
   int reach = 0;                // elements from a stage's start a leaf read may touch
 };
 
+// Who chose a plan's configuration: its own time estimates, a tuning database
+// entry for its geometry, or the caller (select, tune).  A plan made from
+// another one takes over a choice that was made, not an estimate, which is
+// for the other plan's size.
+enum class ChosenBy : int { Estimate = 0, Database = 1, Caller = 2 };
+
 struct TileConfig {
   Kind kind;
   int bd;       // DM trials per block
@@ -273,6 +279,7 @@ struct dd_plan_s {
   std::vector<void*> d_gs;            // GSUM descriptors and their index
   std::vector<dd::TileConfig> configs;
   int selected = 0;
+  dd::ChosenBy chosen_by = dd::ChosenBy::Estimate;  // who chose it
   int fallback = 0;                   // configuration for inputs the selected one cannot take
   // host-buffer forward staging (allocated on first dd_forward_host)
   void* h_dev_in = nullptr;

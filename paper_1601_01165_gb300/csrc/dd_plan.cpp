@@ -647,6 +647,7 @@ extern "C" dd_status dd_plan_select_config(dd_plan_t plan, int32_t k) {
   if (k < 0 || k >= (int32_t)plan->configs.size())
     return set_error(DD_ERR_ARG, "dd_plan_select_config: config %d out of range [0, %zu)", k, plan->configs.size());
   plan->selected = k;
+  plan->chosen_by = ChosenBy::Caller;
   return DD_OK;
 }
 

@@ -4,8 +4,8 @@
 // under a second; Section 2.1 notes that producing s output samples needs
 // s + max_delay input samples.  A stream therefore keeps the last max_delay
 // samples of every channel on the device: chunk k is copied behind that
-// tail, the forward kernel (the plan's tuned configuration, n_out =
-// chunk_len) produces chunk_len outputs starting at absolute time
+// tail, the forward kernel (of a plan of its own with n_out = chunk_len, in the
+// configuration selected or tuned for the caller's plan, if any) produces chunk_len outputs starting at absolute time
 // k*chunk_len - max_delay, and the last max_delay input samples become the
 // next tail.  Two buffers alternate so the tail never overlaps its source.
 #include <cuda_runtime.h>
@@ -47,10 +47,18 @@ extern "C" dd_status dd_stream_create(dd_stream_t* out, dd_plan_t plan, int64_t 
     delete st;
     return s;
   }
-  // keep the caller's kernel choice when the chunk geometry allows it
-  const std::string& want = plan->configs[plan->selected].name;
-  for (size_t k = 0; k < st->chunk_plan->configs.size(); ++k)
-    if (st->chunk_plan->configs[k].name == want) st->chunk_plan->selected = (int)k;
+  // A choice made for the plan (selected, tuned, or found in a tuning database)
+  // holds for its streams, if the chunk geometry allows it; one that a database
+  // has for the chunk geometry itself comes before another entry.  Otherwise the
+  // chunk plan's own estimate stands: the plan's is for its own n_out.
+  if (plan->chosen_by > st->chunk_plan->chosen_by) {
+    const std::string& want = plan->configs[plan->selected].name;
+    for (size_t k = 0; k < st->chunk_plan->configs.size(); ++k)
+      if (st->chunk_plan->configs[k].name == want) {
+        st->chunk_plan->selected = (int)k;
+        st->chunk_plan->chosen_by = plan->chosen_by;
+      }
+  }
   st->n = chunk_len;
   st->max_d = plan->max_delay;
   st->C = plan->C;

@@ -66,7 +66,10 @@ void apply_tune_db(dd_plan_s* plan) {
   double ms = 0;
   if (!db_lookup(path, tune_key(*plan), name, ms)) return;
   for (size_t k = 0; k < plan->configs.size(); ++k)
-    if (plan->configs[k].name == name) plan->selected = (int)k;
+    if (plan->configs[k].name == name) {
+      plan->selected = (int)k;
+      plan->chosen_by = ChosenBy::Database;
+    }
 }
 
 }  // namespace dd
@@ -85,6 +88,7 @@ extern "C" dd_status dd_tune(dd_plan_t plan, double budget_s, const char* db_pat
       for (size_t k = 0; k < plan->configs.size(); ++k)
         if (plan->configs[k].name == name) {
           plan->selected = (int)k;
+          plan->chosen_by = ChosenBy::Caller;
           if (best_ms) *best_ms = ms;
           return DD_OK;
         }
@@ -151,6 +155,7 @@ extern "C" dd_status dd_tune(dd_plan_t plan, double budget_s, const char* db_pat
   clear_error();
   if (best < 0) return set_error(DD_ERR_CUDA, "dd_tune: no configuration ran");
   plan->selected = best;
+  plan->chosen_by = ChosenBy::Caller;
   if (best_ms) *best_ms = med[best];
   if (db_path) {
     FILE* f = std::fopen(db_path, "a");

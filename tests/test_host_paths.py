@@ -1,0 +1,140 @@
+"""Which kernels the library's host code launches, and what it does when memory
+runs out, without a GPU: the library's own objects linked with a CUDA runtime
+that only records launches (fake_cudart.cpp)."""
+import ctypes
+import glob
+import json
+import os
+import subprocess
+
+import pytest
+
+from paper_1601_01165_gb300 import build, synth
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+U8, F32 = 0, 1
+
+
+class Host:
+    """The library on the recording runtime."""
+
+    def __init__(self, path):
+        lib = self.lib = ctypes.CDLL(path)
+        i32, i64, dbl, vp = ctypes.c_int32, ctypes.c_int64, ctypes.c_double, ctypes.c_void_p
+        lib.dd_plan.argtypes = [ctypes.POINTER(vp), i32, dbl, dbl, dbl, dbl, dbl, i32, i64, ctypes.c_int]
+        lib.dd_plan_config_name.argtypes, lib.dd_plan_config_name.restype = [vp, i32], ctypes.c_char_p
+        lib.dd_plan_select_config.argtypes = [vp, i32]
+        lib.dd_plan_selected_config.argtypes = [vp, ctypes.POINTER(i32)]
+        lib.dd_plan_num_configs.argtypes = [vp, ctypes.POINTER(i32)]
+        lib.dd_plan_destroy.argtypes = [vp]
+        lib.dd_tune.argtypes = [vp, dbl, ctypes.c_char_p, ctypes.POINTER(dbl)]
+        lib.dd_forward.argtypes = [vp, vp, i64, vp, vp, i64, vp]
+        lib.dd_plan_in_stride.argtypes = [vp, ctypes.POINTER(i64)]
+        lib.dd_stream_create.argtypes = [ctypes.POINTER(vp), vp, i64]
+        lib.dd_stream_push.argtypes = [vp, vp, vp, ctypes.POINTER(i64), vp]
+        lib.dd_stream_destroy.argtypes = [vp]
+        lib.fake_launch_name.restype = ctypes.c_char_p
+
+    def plan(self, setup, dtype):
+        h = ctypes.c_void_p()
+        assert self.lib.dd_plan(ctypes.byref(h), *setup.plan_args(), dtype) == 0
+        return h
+
+    def configs(self, h):
+        n = ctypes.c_int32()
+        self.lib.dd_plan_num_configs(h, ctypes.byref(n))
+        return [self.lib.dd_plan_config_name(h, k).decode() for k in range(n.value)]
+
+    def selected(self, h):
+        k = ctypes.c_int32()
+        self.lib.dd_plan_selected_config(h, ctypes.byref(k))
+        return self.configs(h)[k.value]
+
+    def launches(self, call):
+        self.lib.fake_clear_launches()
+        assert call() == 0
+        return [self.lib.fake_launch_name(k).decode() for k in range(self.lib.fake_launches())]
+
+    def forward(self, h):
+        stride = ctypes.c_int64()
+        self.lib.dd_plan_in_stride(h, ctypes.byref(stride))
+        return self.launches(lambda: self.lib.dd_forward(h, 4096, stride.value, None, 8192, 1 << 30, None))
+
+    def push(self, h, chunk):
+        """The kernels one push into a stream made from the plan launches."""
+        st, t0 = ctypes.c_void_p(), ctypes.c_int64()
+        assert self.lib.dd_stream_create(ctypes.byref(st), h, chunk) == 0
+        names = self.launches(lambda: self.lib.dd_stream_push(st, 4096, 8192, ctypes.byref(t0), None))
+        self.lib.dd_stream_destroy(st)
+        return names
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    build.build()
+    out = str(tmp_path_factory.mktemp("host") / "libdd_host.so")
+    objs = sorted(glob.glob(os.path.join(build.BUILD, "*.o")))
+    subprocess.run(["g++", "-shared", "-fPIC", "-O1", "-o", out, os.path.join(HERE, "fake_cudart.cpp"), *objs,
+                    "-Wl,--no-undefined", "-lpthread", "-ldl"], check=True)
+    return Host(out)
+
+
+def _apertif(n_out, n_dm=2048, C=1024):
+    return synth.Setup("host", C, 1420.0, 300.0 / C, 50e-6, 0.0, 0.25, n_dm, n_out)
+
+
+# ------------------------------------------------------------------ streams
+@pytest.mark.parametrize("dtype", [F32, U8], ids=["f32", "u8"])
+@pytest.mark.parametrize("n_dm", [64, 512])
+@pytest.mark.parametrize("chunk", [500, 20000])
+def test_a_stream_chooses_for_its_chunks(host, dtype, n_dm, chunk):
+    """Whatever the plan's n_out: a push runs the kernel that a forward call of the chunk's length would."""
+    want = host.forward(host.plan(_apertif(chunk, n_dm), dtype))
+    for n_out in (1, 256, 1000, 20000):
+        assert host.push(host.plan(_apertif(n_out, n_dm), dtype), chunk) == want, n_out
+
+
+@pytest.mark.parametrize("dtype", [F32, U8], ids=["f32", "u8"])
+def test_a_stream_keeps_what_was_selected(host, dtype):
+    for name in host.configs(host.plan(_apertif(1, 64), dtype)):
+        chunk_plan = host.plan(_apertif(3000, 64), dtype)
+        host.lib.dd_plan_select_config(chunk_plan, host.configs(chunk_plan).index(name))
+        want = host.forward(chunk_plan)
+        h = host.plan(_apertif(1, 64), dtype)
+        host.lib.dd_plan_select_config(h, host.configs(h).index(name))
+        assert host.push(h, 3000) == want, name
+    h = host.plan(_apertif(1, 64), dtype)
+    assert host.lib.dd_tune(h, 0.0, None, None) == 0     # every time the same here: the most promising one
+    name = host.selected(h)
+    chunk_plan = host.plan(_apertif(3000, 64), dtype)
+    host.lib.dd_plan_select_config(chunk_plan, host.configs(chunk_plan).index(name))
+    assert host.push(h, 3000) == host.forward(chunk_plan)
+
+
+def test_a_stream_and_the_tuning_database(host, tmp_path, monkeypatch):
+    """An entry for the plan holds for its streams, unless there is one for the chunks' own length; a selection wins."""
+    def key(n_out):
+        s = _apertif(n_out, 64)
+        return (f"fake|C={s.channels}|f_low=1420|chan_bw={s.chan_bw_mhz:.9g}|t_samp=5e-05|dm_first=0|dm_step=0.25|"
+                f"n_dm=64|n_out={n_out}|f32")
+
+    def entry(n_out, name):
+        return json.dumps({"key": key(n_out), "config": name, "ms": 1.0}) + "\n"
+
+    db = tmp_path / "tune.jsonl"
+    monkeypatch.setenv("DD_TUNE_DB", str(db))
+
+    def kernel(name):
+        h = host.plan(_apertif(777, 64), F32)
+        host.lib.dd_plan_select_config(h, host.configs(h).index(name))
+        return host.forward(h)
+
+    db.write_text(entry(1000, "staged_d64_t256_c4_s3"))
+    h = host.plan(_apertif(1000, 64), F32)
+    assert host.selected(h) == "staged_d64_t256_c4_s3"
+    assert host.push(h, 3000) == kernel("staged_d64_t256_c4_s3")
+    db.write_text(entry(1000, "staged_d64_t256_c4_s3") + entry(3000, "naive_t32"))
+    h = host.plan(_apertif(1000, 64), F32)
+    assert host.push(h, 3000) == kernel("naive_t32")
+    host.lib.dd_plan_select_config(h, host.configs(h).index("staged_d16_t256_c8_s3"))
+    assert host.push(h, 3000) == kernel("staged_d16_t256_c8_s3")
