@@ -39,56 +39,84 @@ struct AccOf<uint8_t> {
 // ------------------------------------------------------------------ NAIVE
 
 // What bounds it on the small launches it is chosen for is the latency of one
-// load after another down the channels, so kNaiveBatch channels' delays, then
-// their samples, are all in flight before the first is added (in channel
-// order, as everywhere).
-constexpr int kNaiveBatch = 16;
+// load after another down the channels, so a batch of channels' delays, then
+// their samples, are in flight before the first is added (in channel order, as
+// everywhere).  Large launches are bound by instructions: the row pointer is
+// incremented, not multiplied out per load.  Against one load after another
+// (us; a multiplied-out batch of 16 for both types in brackets):
+//                                   float             uint8
+//   1024 x 16 x 3000                80 -> 23 (33)     49 -> 32 (31)
+//   1024 x 512 x 20,000             4910 -> 3210 (3820)  3190 -> 3200 (3530)
+//   LOFAR 32 x 1024 x 50,000        628 -> 551 (664)  504 -> 493 (608)
+//   LOFAR 319 x 750 x 6048, steep   779 -> 666 (582)  506 -> 491 (534)
+// Float reads the next batch's delays while a batch's samples are on their way
+// (without: 44 us on the smallest); uint8, which that slows (42 us), takes 32.
+// With weights the multiplied-out form is the faster one (1024 x 16 x 3000: 47
+// against 90 us, 1024 x 512 x 20,000: 4930 against 7090).
+template <typename Tin>
+struct NaiveBatch {
+  static constexpr int kN = sizeof(Tin) == 1 ? 32 : 16;
+  static constexpr bool kAhead = sizeof(Tin) != 1;
+};
 
 template <typename Tin, bool WEIGHTED>
 __global__ void __launch_bounds__(256) fwd_naive_kernel(FwdArgs a) {
   using Tacc = typename AccOf<Tin>::type;
-  const Tin* __restrict__ in = static_cast<const Tin*>(a.in);
+  constexpr int N = NaiveBatch<Tin>::kN;
+  constexpr bool kAhead = NaiveBatch<Tin>::kAhead;
   Tacc* __restrict__ out = static_cast<Tacc*>(a.out);
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= a.n_out) return;
   for (int64_t i = blockIdx.y; i < a.n_dm; i += gridDim.y) {
     const int32_t* __restrict__ drow = a.delays + i * a.C;
-    const Tin* __restrict__ col = in + t;
+    const Tin* __restrict__ row = static_cast<const Tin*>(a.in) + t;  // of channel c (weighted: of the first)
     Tacc acc = 0;
-    int c = 0;
-    int32_t d[kNaiveBatch];
-    if (a.C >= kNaiveBatch) {
-#pragma unroll
-      for (int k = 0; k < kNaiveBatch; ++k) d[k] = __ldg(drow + k);
-    }
-    for (; c + kNaiveBatch <= a.C; c += kNaiveBatch) {
-      Tin v[kNaiveBatch];
-      float w[kNaiveBatch];
+    auto add = [&](Tin v, float w) {
       if constexpr (WEIGHTED) {
-#pragma unroll
-        for (int k = 0; k < kNaiveBatch; ++k) w[k] = __ldg(a.w + c + k);
-      }
-#pragma unroll
-      for (int k = 0; k < kNaiveBatch; ++k) v[k] = __ldg(col + (int64_t)(c + k) * a.in_stride + d[k]);
-      if (c + 2 * kNaiveBatch <= a.C) {
-#pragma unroll
-        for (int k = 0; k < kNaiveBatch; ++k) d[k] = __ldg(drow + c + kNaiveBatch + k);
-      }
-#pragma unroll
-      for (int k = 0; k < kNaiveBatch; ++k) {
-        if constexpr (WEIGHTED) {
-          acc = fmaf(w[k], v[k], acc);
-        } else {
-          acc += (Tacc)v[k];
-        }
-      }
-    }
-    for (; c < a.C; ++c) {
-      const Tin v = __ldg(col + (int64_t)c * a.in_stride + __ldg(drow + c));
-      if constexpr (WEIGHTED) {
-        acc = fmaf(__ldg(a.w + c), v, acc);
+        acc = fmaf(w, v, acc);
       } else {
         acc += (Tacc)v;
+      }
+    };
+    int c = 0;
+    int32_t d[N];
+    if (kAhead && a.C >= N) {
+#pragma unroll
+      for (int k = 0; k < N; ++k) d[k] = __ldg(drow + k);
+    }
+    for (; c + N <= a.C; c += N) {
+      Tin v[N];
+      float w[N] = {};
+      if constexpr (WEIGHTED) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) w[k] = __ldg(a.w + c + k);
+      }
+      if constexpr (!kAhead) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) d[k] = __ldg(drow + c + k);
+      }
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        if constexpr (WEIGHTED) {
+          v[k] = __ldg(row + (int64_t)(c + k) * a.in_stride + d[k]);
+        } else {
+          v[k] = __ldg(row + d[k]);
+          row += a.in_stride;
+        }
+      }
+      if (kAhead && c + 2 * N <= a.C) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) d[k] = __ldg(drow + c + N + k);
+      }
+#pragma unroll
+      for (int k = 0; k < N; ++k) add(v[k], w[k]);
+    }
+    for (; c < a.C; ++c) {
+      if constexpr (WEIGHTED) {
+        add(__ldg(row + (int64_t)c * a.in_stride + __ldg(drow + c)), __ldg(a.w + c));
+      } else {
+        add(__ldg(row + __ldg(drow + c)), 1.0f);
+        row += a.in_stride;
       }
     }
     out[i * a.out_stride + t] = acc;
