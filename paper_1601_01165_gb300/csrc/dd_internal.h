@@ -43,6 +43,7 @@ struct GsLaunch {
   int padp = 0;                 // staged row pitch less the tile length
   int cap = 0;                  // row elements of one of the two buffers
   float patterns = 0;           // patterns per block and group, on average
+  float samples = 0;            // samples of their rows, likewise
   int reach = 0;                // elements from a stage's start a leaf read may touch
 };
 
@@ -169,15 +170,19 @@ int64_t tmw9_min_in_stride(int64_t n_in);
 struct GsTable {
   int padp = 0, desc_max = 0;
   int64_t cap = 0;                                // row elements one buffer needs
-  int64_t patterns = 0;             // over all (trial block, channel group) pairs
+  int64_t patterns = 0, samples = 0;  // over all (trial block, channel group) pairs
   std::vector<uint2> idx;
   std::vector<uint4> desc;
   size_t idx_bytes() const { return idx.size() * sizeof(uint2); }
   size_t desc_bytes() const { return desc.size() * sizeof(uint4); }
 };
 bool gsum_build(const dd_plan_s& p, int bd, int T, GsTable& t);
-// Patterns per block of `bd` trials and group, on a sample of them (-1: no descriptors).
-double gsum_patterns(const dd_plan_s& p, int bd);
+// Patterns per block of `bd` trials and group, and samples of their rows in
+// tiles of T, on a sample of them (patterns < 0: no descriptors).
+struct GsSample {
+  double patterns, samples;
+};
+GsSample gsum_sample(const dd_plan_s& p, int bd, int T);
 int gsum_smem_for(dd_dtype dtype, const TileConfig& cfg);
 int32_t block_spread_of(const dd_plan_s& p, int bd);
 

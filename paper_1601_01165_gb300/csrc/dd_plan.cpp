@@ -158,9 +158,10 @@ static GsumTables gsum_tables(const dd_plan_s& p) {
     for (TileConfig cfg : gsum_menu(p.dtype)) {
       const double most = gs_max_patterns(p, cfg);
       if (most <= 0.0) continue;
-      const double patterns = gsum_patterns(p, cfg.bd);
-      if (patterns < 0.0 || patterns > most) continue;
-      cfg.gs.patterns = (float)patterns;
+      const GsSample s = gsum_sample(p, cfg.bd, cfg.bt);
+      if (s.patterns < 0.0 || s.patterns > most) continue;
+      cfg.gs.patterns = (float)s.patterns;
+      cfg.gs.samples = (float)s.samples;
       // the adjoint's plan is made by the first call that needs it: only a table it will use
       if (p.grouped && estimate_us(p, cfg) >= estimate_us(p, p.configs[best_config(p, false)])) continue;
       GsTable t;
@@ -241,11 +242,13 @@ void free_plan_device(dd_plan_s* p) {
 // Default configuration: the one whose time estimate is least.  The launch sizes
 // decide between the kernels (40 tiles of TMW9 leave most SMs idle, and short
 // chains of plain loads beat them), so the estimate is what was measured of
-// each on this GPU, in microseconds per channel:
-//   waves x (time of a block that shares its SM with as many as fit), but no
+// each on this GPU (hence its 152 SMs, wherever the estimate is made), in
+// microseconds per channel:
+//   waves x (time of a block that shares its SM with as many as fill it), but no
 //   less than the time of a block alone, plus what a launch costs.
 //                      wave   alone   measured on (channels x trials x samples)
 //   tmw9               0.303  0.303   1024 x 2048 x 20,000: 2.49 ms; x 64: 316 us
+//   tmw6               0.331  0.331   1024 x 2048 x 20,000: 4.07 ms
 //   staged d32 t512 c8 0.285  0.385   LOFAR beam 3.07 ms (d8 t1024 3.15); 107 x 2947 x 6576: 253 us
 //   staged d16 t512    0.156  0.27    403 x 89 x 21,373: 140 us
 //   staged d8 t1024    0.149  0.31    171 x 449 x 47,040: 478 us (d32 513)
@@ -253,38 +256,61 @@ void free_plan_device(dd_plan_s* p) {
 //   staged d8 t256     0.046  0.155   768 x 251 x 2414: 142 us (tmw9 239)
 //   u8pk 32 trials     0.165  0.257   and 3.8 us per million outputs and 256 channels (its sums leave by
 //                                     reading the output back): LOFAR 256 x 1024 x 50,000 650 us (16 trials 873)
-//   u8pk 16 trials     0.112  0.142   167 x 1618 x 27,087: 414 us (32 trials 487)
+//   u8pk 16 trials     0.108  0.142   167 x 1618 x 27,087: 414 us (32 trials 487); 16-channel chunks 0.112, 0.150
+//   u8pk 1792 samples  0.11   0.149
 //   u8pk 8 trials      0.075  0.104   182 x 92 x 5295: 23 us (16 trials 31)
 // A staged wave costs the more the fewer there are (the ends of blocks overlap
-// less), u8pk 1.25 times as much where long spans leave one block an SM, and 32
-// trials only pay from eight waves on (281 x 212 x 36,563: 254 us, 16 trials 165).
-// The plain kernel needs 0.030 a channel, or 2.4 T adds/s where that is more
-// (1024 x 16 x 3000: 33 us, tmw9 311, staged 158).
-// GSUM's times grow with the patterns its blocks have (13.7 and 8.7 on the
-// Apertif beam): 64 trials 1.39 ms there (u8pk 2.09), 32 trials 98 us on
-// 1024 x 64 x 20,000 (u8pk 145), 16 trials 75 us on 768 x 251 x 2414 (u8pk 85);
-// float, on the Apertif beam's adjoint: 3.4 ms (staged 7.1).
+// less), u8pk 32 trials 1.25 times as much where long spans leave one block an SM, and
+// only pay from eight waves on (281 x 212 x 36,563: 254 us, 16 trials 165).
+// Steep grids have spans much longer than their tiles.  What they cost is not the
+// longer copies but the blocks that no longer fit an SM together: with one, each
+// takes its own time (staged d8 t1024 0.30 a wave at any span from 9 to 17 KB,
+// uint8 and float), with a few a little more than their share of it.  Timed on
+// 1,020 random beams at 0 to 256 times the surveys' DM steps, the choice is
+// within 2 % of the best of the menu on average and within 5 % of the fixed
+// preference list it replaced on every one (LOFAR 30 x 477 x 66,978 at 0.32, uint8:
+// staged d8 t1024 161 us, plain 445; Apertif 447 x 223 x 17,992 at 8, float:
+// 325 us, d8 t512 553).
+// The plain kernel needs 0.030 a channel (uint8; float less), or 2.4 T adds/s where
+// that is more, with eight channels' worth of time for each output (float LOFAR
+// 319 x 750 x 6048 at 0.64: 530 us in blocks of 256, 666 in blocks of 128; 1024 x 2 x
+// 20,000: 49 and 26).
+// GSUM's times grow with the samples of the rows its blocks make (a block's
+// patterns times the row's length; 11,000 a group on the Apertif beam), which the
+// row makers may need longer for than the adding: 64 trials 1.39 ms there (u8pk 2.09),
+// 32 trials 98 us on 1024 x 64 x 20,000 (u8pk 145), 16 trials 75 us on
+// 768 x 251 x 2414 (u8pk 85); float, on the Apertif beam's adjoint: 3.4 ms (staged 7.1).
 static double estimate_us(const dd_plan_s& p, const TileConfig& c) {
   constexpr double kNever = 1e30;
   const double C = p.C, outputs = p.n_dm * (double)p.n_out;
   const double tiles = std::ceil((double)p.n_dm / c.bd) * std::ceil((double)p.n_out / c.bt);
   const double waves = std::ceil(tiles / 152.0);
   auto time = [&](double wave, double alone) { return 6.0 + C * std::max(alone, waves * wave); };
+  // blocks whose spans fit an SM together: fewer than it takes to fill its time
+  // cost a block's own time each
+  const double fit = std::max(1.0, std::floor(228.0 * 1024 / (c.smem + 1024)));
+  auto spans = [&](double wave, double alone) {
+    return time(std::max(wave, fit > 1.0 ? 1.15 * alone / fit : alone), alone);
+  };
   const bool u8 = p.dtype == DD_U8_I32;
   switch (c.kind) {
     case Kind::Naive:
-      if (c.threads != 128) return kNever;
-      return 5.0 + std::max(0.030 * C, C * outputs / 2.4e6);
+      // (launches of more threads than fit the SMs at once: blocks of 256, the same
+      // on 200 random ones on average, 5 to 20 % less on steep float ones of many
+      // channels; small ones up to 1.9 times as much)
+      if (c.threads != (outputs > 152.0 * 2048 ? 256 : 128)) return kNever;
+      return 5.0 + std::max(0.030 * C, (C + 8.0) * outputs / 2.4e6);
     case Kind::TmW9:
       return 1.0 + time(0.303, 0.303);
+    case Kind::TmW6:
+      return 1.0 + time(0.331, 0.331);
     case Kind::Staged:
-      if (u8) return kNever;
-      if (c.bd == 32 && c.bt == 512 && c.cc == 8) return time(0.285 + 0.086 / waves, 0.385);
-      if (c.bd == 16 && c.bt == 512) return time(0.156 + 0.078 / waves, 0.27);
-      if (c.bd == 8 && c.bt == 1024) return time(0.149 + 0.042 / waves, 0.31);
-      if (c.bd == 8 && c.bt == 512) return time(0.078 + 0.057 / waves, 0.187);
+      if (c.bd == 32 && c.bt == 512 && c.cc == 8 && !u8) return spans(0.285 + 0.086 / waves, 0.385);
+      if (c.bd == 16 && c.bt == 512) return spans(0.156 + 0.078 / waves, 0.27);
+      if (c.bd == 8 && c.bt == 1024) return spans(0.149 + 0.042 / waves, 0.31);
+      if (c.bd == 8 && c.bt == 512) return spans(0.078 + 0.057 / waves, 0.187);
       if (c.bd == 8 && c.bt == 256)  // long spans cost its short tiles most (293 x 1081 x 1064, LOFAR: 0.067)
-        return time((0.046 + 0.045 / waves) * (1.0 + 0.22 * (c.pitch - c.bt) / c.bt), 0.155);
+        return spans((0.046 + 0.045 / waves) * (1.0 + 0.22 * (c.pitch - c.bt) / c.bt), 0.155);
       return kNever;
     case Kind::U8Pk: {
       const double one = 2 * (c.smem + 1024) > 228 * 1024 ? 1.25 : 1.0;  // one block an SM
@@ -292,17 +318,25 @@ static double estimate_us(const dd_plan_s& p, const TileConfig& c) {
         return waves < 8.0 ? kNever
                            : time(0.165 * one * (c.cc == 16 ? 1.03 : 1.0), 0.257) +
                                  3.8e-6 * outputs * std::ceil(C / 256.0);
-      if (c.bd == 16 && c.cc == 32) return time(0.112 * one, 0.142) + 0.5e-6 * outputs;
+      if (c.bd == 16 && c.bt == 896) return spans(c.cc == 32 ? 0.108 : 0.112, c.cc == 32 ? 0.142 : 0.150) + 0.6e-6 * outputs;
+      if (c.bt == 1792) return spans(c.bd == 8 && c.threads == 512 ? 0.115 : 0.11, 0.149) + 0.85e-6 * outputs;
       if (c.bd == 8 && c.threads == 128)  // two blocks an SM
-        return time(0.15 * std::ceil(waves / 2.0) / waves, 0.104) + 0.5e-6 * outputs;
+        return spans(0.15 * std::ceil(waves / 2.0) / waves, 0.104) + 0.5e-6 * outputs;
       return kNever;
     }
-    case Kind::GSum:
+    case Kind::GSum: {
+      if (c.gs.patterns > 0.9 * std::min(c.bd, p.n_dm)) return kNever;  // hardly two trials share one
       if (!u8) return time(0.12 + 0.0065 * c.gs.patterns, 0.20);
-      if (c.bd == 64 && c.bt == 576) return time(0.062 + 0.0078 * c.gs.patterns, 0.150);
-      if (c.bd == 64) return time(0.047 + 0.0065 * c.gs.patterns, 0.121);
-      if (c.bd == 32) return time(0.053 + 0.0047 * c.gs.patterns, 0.0);
-      return time(0.038 + 0.0035 * c.gs.patterns, 0.085);
+      const double rows = 1e-3 * c.gs.samples;  // thousands of row samples a group
+      // adding the rows up; making them, if that takes longer; a block alone
+      auto gsum = [&](double add, double make, double alone) {
+        return 6.0 + C * std::max({waves * add, std::ceil(waves / (c.bd == 16 ? 2.0 : 1.0)) * make * rows, alone});
+      };
+      if (c.bd == 64 && c.bt == 576) return gsum(0.085 + 0.0090 * rows, 0.0163, 0.103);
+      if (c.bd == 64) return gsum(0.088 + 0.0059 * rows, 0.0149, 0.098);
+      if (c.bd == 32) return gsum(0.079 + 0.0029 * rows, 0.0152, 0.083);
+      return gsum(0.044 + 0.0065 * rows, 0.0293, 0.080);
+    }
     default:
       return kNever;
   }
@@ -316,7 +350,7 @@ std::vector<int> config_preference_order(const dd_plan_s& p) {
     order[j] = (int)j;
     est[j] = estimate_us(p, p.configs[j]);
     // the plain kernel's other block sizes last
-    if (p.configs[j].kind == Kind::Naive && p.configs[j].threads != 128) est[j] *= 2.0;
+    if (p.configs[j].kind == Kind::Naive && est[j] >= 1e30) est[j] *= 2.0;
   }
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return est[x] < est[y]; });
   return order;

@@ -84,6 +84,7 @@ static void build_blocks(const dd_plan_s& p, int bd, int T, int padp, int b0, in
       const int row_len = (T + e[bd - 1] + chunk - 1) / chunk * chunk;
       t.cap = std::max<int64_t>(t.cap, (int64_t)n_p * row_len);
       t.patterns += n_p;
+      t.samples += (int64_t)n_p * row_len;
       const size_t at = t.desc.size();
       t.desc.resize(at + 1 + bd / 4);
       uint32_t* tr = reinterpret_cast<uint32_t*>(&t.desc[at + 1]);
@@ -139,17 +140,17 @@ static int pitch_pad(const dd_plan_s& p, int bd) {
   return pad > 4000 ? -1 : (int)pad;  // (keys of 13 bits, staged byte offsets below 2^24)
 }
 
-double gsum_patterns(const dd_plan_s& p, int bd) {
+GsSample gsum_sample(const dd_plan_s& p, int bd, int T) {
   const int pad = pitch_pad(p, bd);
-  if (pad < 0) return -1.0;
+  if (pad < 0) return {-1.0, 0.0};
   GsTable t;
   // (whole blocks: a last one of few trials has few patterns but takes as long)
   const int n_b = std::max(1, p.n_dm / bd), n_g = (p.C + kGsGroup - 1) / kGsGroup;
   for (int k = 0; k < 4; ++k) {
     const int b = (int)((int64_t)k * n_b / 4);
-    build_blocks(p, bd, 512, pad, b, b + 1, std::max(1, n_g / 16), t);
+    build_blocks(p, bd, T, pad, b, b + 1, std::max(1, n_g / 16), t);
   }
-  return (double)t.patterns / (double)t.idx.size();
+  return {(double)t.patterns / (double)t.idx.size(), (double)t.samples / (double)t.idx.size()};
 }
 
 bool gsum_build(const dd_plan_s& p, int bd, int T, GsTable& t) {

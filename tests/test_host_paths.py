@@ -138,3 +138,36 @@ def test_a_stream_and_the_tuning_database(host, tmp_path, monkeypatch):
     assert host.push(h, 3000) == kernel("naive_t32")
     host.lib.dd_plan_select_config(h, host.configs(h).index("staged_d16_t256_c8_s3"))
     assert host.push(h, 3000) == kernel("staged_d16_t256_c8_s3")
+
+
+# ------------------------------------------------------- choice on steep grids
+# (band, channels, trials, samples, DM step; the configurations within 15 % of
+# the fastest of the menu as timed on the GPU, fastest first)
+STEEP = [
+    ("lofar", 30, 477, 66978, 0.32, U8, ["staged_d8_t1024_c4_s3"]),                       # 161 us; plain 445
+    ("lofar", 18, 242, 81259, 0.32, U8, ["staged_d8_t1024_c4_s3"]),                       # 66; 181
+    ("apertif", 521, 257, 17780, 16.0, U8, ["u8pk_w4x2_d2_c16_st4", "u8pk_w8x2_d1_c16_st4"]),  # 244; 811
+    ("apertif", 389, 179, 41677, 64.0, U8, ["staged_d8_t1024_c4_s3"]),                    # 535; 991
+    ("lofar", 23, 1455, 25939, 0.01, U8, ["u8pk_w8x1_d2_c16_st4"]),                       # 76; 32-channel chunks 103
+    ("apertif", 447, 223, 17992, 8.0, F32, ["staged_d8_t1024_c4_s3"]),                    # 325; d8 t512 553
+    ("lofar", 229, 458, 16729, 0.04, F32, ["staged_d8_t1024_c4_s3"]),                     # 309; d8 t512 529
+    ("apertif", 52, 3471, 8917, 4.0, F32, ["staged_d8_t1024_c4_s3"]),                     # 212; d32 t512 277
+    ("lofar", 766, 6, 2812, 0.64, U8, ["naive_t128"]),                                    # 19; staged 238
+    ("lofar", 449, 55, 2424, 0.02, F32, ["naive_t128"]),                                  # 29; staged 140
+]
+
+
+@pytest.mark.parametrize("band,C,n_dm,n_out,step,dtype,good", STEEP)
+def test_default_on_steep_grids(host, band, C, n_dm, n_out, step, dtype, good):
+    f_low, bw, t_samp = {"apertif": (1420.0, 300.0, 50e-6), "lofar": (138.0, 6.25, 5e-6)}[band]
+    assert host.selected(host.plan(synth.Setup("steep", C, f_low, bw / C, t_samp, 0.0, step, n_dm, n_out), dtype)) in good
+
+
+@pytest.mark.parametrize("C,n_dm,n_out,step", [(460, 641, 18008, 0.25), (753, 118, 21229, 2.0)])
+def test_adjoint_too_steep_for_nine_trials_takes_six(host, C, n_dm, n_out, step):
+    """705 and 244 us with six-trial windows; staged 841 and 279."""
+    i64, vp = ctypes.c_int64, ctypes.c_void_p
+    host.lib.dd_adjoint.argtypes = [vp, vp, i64, vp, vp, i64, vp, i64, vp, vp]
+    h = host.plan(synth.Setup("steep", C, 1420.0, 300.0 / C, 50e-6, 0.0, step, n_dm, n_out), F32)
+    names = host.launches(lambda: host.lib.dd_adjoint(h, 4096, 1 << 40, None, 8192, 1 << 40, None, 0, None, None))
+    assert len(names) == 1 and "fwd_tmw6_kernel" in names[0], names
