@@ -75,7 +75,7 @@ def host(tmp_path_factory):
     out = str(tmp_path_factory.mktemp("host") / "libdd_host.so")
     objs = sorted(glob.glob(os.path.join(build.BUILD, "*.o")))
     subprocess.run(["g++", "-shared", "-fPIC", "-O1", "-o", out, os.path.join(HERE, "fake_cudart.cpp"), *objs,
-                    "-Wl,--no-undefined", "-lpthread", "-ldl"], check=True)
+                    "-Wl,--no-undefined", "-Wl,-Bsymbolic", "-lpthread", "-ldl"], check=True)
     return Host(out)
 
 
