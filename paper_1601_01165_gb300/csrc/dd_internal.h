@@ -165,24 +165,27 @@ bool tmw6_accepts(const void* in, int64_t in_stride);
 bool tmw9_accepts(const void* in, int64_t in_stride, int64_t n_in);
 int64_t tmw9_min_in_stride(int64_t n_in);
 
-// Host form of a plan's GSUM descriptors for blocks of `bd` trials
-// (gsum_plan.cpp); false if the plan's delays do not fit them.
+// Host form of a plan's GSUM descriptors for blocks of `bd` trials and tiles of T
+// samples (gsum_plan.cpp); `fits` unless the plan's delays are beyond them.
 struct GsTable {
+  int bd = 0, T = 0;
+  bool fits = false;
   int padp = 0, desc_max = 0;
-  int64_t cap = 0;                                // row elements one buffer needs
+  int64_t cap = 0;                    // row elements one buffer needs
   int64_t patterns = 0, samples = 0;  // over all (trial block, channel group) pairs
   std::vector<uint2> idx;
   std::vector<uint4> desc;
   size_t idx_bytes() const { return idx.size() * sizeof(uint2); }
   size_t desc_bytes() const { return desc.size() * sizeof(uint4); }
 };
-bool gsum_build(const dd_plan_s& p, int bd, int T, GsTable& t);
+void gsum_build(const dd_plan_s& p, std::vector<GsTable>& tables);  // (each with its bd and T)
 // Patterns per block of `bd` trials and group, and samples of their rows in
-// tiles of T, on a sample of them (patterns < 0: no descriptors).
+// tiles of T, on a sample of them, smaller where there are more than twice
+// `most` patterns (patterns < 0: no descriptors).
 struct GsSample {
   double patterns, samples;
 };
-GsSample gsum_sample(const dd_plan_s& p, int bd, int T);
+GsSample gsum_sample(const dd_plan_s& p, int bd, int T, double most);
 int gsum_smem_for(dd_dtype dtype, const TileConfig& cfg);
 int32_t block_spread_of(const dd_plan_s& p, int bd);
 

@@ -155,17 +155,27 @@ static GsumTables gsum_tables(const dd_plan_s& p) {
   GsumTables v;
   if (p.dtype == DD_F32_F32 && !p.grouped) return v;
   try {
+    std::vector<TileConfig> cfgs;
+    std::vector<GsTable> tables;
     for (TileConfig cfg : gsum_menu(p.dtype)) {
       const double most = gs_max_patterns(p, cfg);
       if (most <= 0.0) continue;
-      const GsSample s = gsum_sample(p, cfg.bd, cfg.bt);
+      const GsSample s = gsum_sample(p, cfg.bd, cfg.bt, most);
       if (s.patterns < 0.0 || s.patterns > most) continue;
       cfg.gs.patterns = (float)s.patterns;
       cfg.gs.samples = (float)s.samples;
       // the adjoint's plan is made by the first call that needs it: only a table it will use
       if (p.grouped && estimate_us(p, cfg) >= estimate_us(p, p.configs[best_config(p, false)])) continue;
-      GsTable t;
-      if (!gsum_build(p, cfg.bd, cfg.bt, t)) continue;
+      cfgs.push_back(cfg);
+      tables.emplace_back();
+      tables.back().bd = cfg.bd;
+      tables.back().T = cfg.bt;
+    }
+    if (!tables.empty()) gsum_build(p, tables);
+    for (size_t k = 0; k < tables.size(); ++k) {
+      TileConfig& cfg = cfgs[k];
+      GsTable& t = tables[k];
+      if (!t.fits) continue;
       const int es = p.dtype == DD_U8_I32 ? 1 : 4, er = p.dtype == DD_U8_I32 ? 2 : 4;
       cfg.gs.padp = t.padp;
       cfg.gs.desc_max = t.desc_max;

@@ -171,3 +171,19 @@ def test_adjoint_too_steep_for_nine_trials_takes_six(host, C, n_dm, n_out, step)
     h = host.plan(synth.Setup("steep", C, 1420.0, 300.0 / C, 50e-6, 0.0, step, n_dm, n_out), F32)
     names = host.launches(lambda: host.lib.dd_adjoint(h, 4096, 1 << 40, None, 8192, 1 << 40, None, 0, None, None))
     assert len(names) == 1 and "fwd_tmw6_kernel" in names[0], names
+
+
+# ------------------------------------------------------------------- memory
+@pytest.mark.parametrize("C,n_dm", [(192, 1), (193, 3), (250, 64), (1000, 65), (1024, 255), (1024, 512), (700, 130)])
+def test_footprint_is_what_a_plan_holds(host, C, n_dm):
+    """With the grouped-sum tables of every shape the plan offers."""
+    i32, i64, dbl = ctypes.c_int32, ctypes.c_int64, ctypes.c_double
+    s = _apertif(3000, n_dm, C)
+    host.lib.dd_plan_footprint.argtypes = [i32, dbl, dbl, dbl, dbl, dbl, i32, ctypes.c_int, ctypes.POINTER(i64)]
+    host.lib.dd_plan_info.argtypes = [ctypes.c_void_p, ctypes.POINTER(i64), ctypes.POINTER(i32), ctypes.POINTER(i64)]
+    sized, held = i64(), i64()
+    assert host.lib.dd_plan_footprint(*s.plan_args()[:7], U8, ctypes.byref(sized)) == 0
+    h = host.plan(s, U8)
+    assert C < 1000 or any(c.startswith("gsum8") for c in host.configs(h))
+    host.lib.dd_plan_info(h, None, None, ctypes.byref(held))
+    assert sized.value == held.value
