@@ -474,15 +474,18 @@ dd_status finish_plan(dd_plan_s* p) {
     void* d[2] = {nullptr, nullptr};
     const void* h[2] = {t.idx.data(), t.desc.data()};
     const size_t n[2] = {t.idx_bytes(), t.desc_bytes()};
-    for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
-      e = cudaMalloc(&d[k], n[k]);
-      if (e == cudaSuccess) p->d_gs.push_back(d[k]);
-      if (e == cudaSuccess) e = cudaMemcpy(d[k], h[k], n[k], cudaMemcpyHostToDevice);
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaMalloc(&d[k], n[k]);
+    if (e == cudaErrorMemoryAllocation) {  // the plan works without
+      cudaGetLastError();
+      cudaFree(d[0]);
+      e = cudaSuccess;
+      continue;
     }
+    p->d_gs.insert(p->d_gs.end(), d, d + 2);
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaMemcpy(d[k], h[k], n[k], cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
       free_plan_device(p);
-      return e == cudaErrorMemoryAllocation ? set_error(DD_ERR_NOMEM, "dd_plan: device allocation failed")
-                                            : set_cuda_error("dd_plan: upload", e);
+      return set_cuda_error("dd_plan: upload", e);
     }
     p->device_bytes += (int64_t)(n[0] + n[1]);
     cfg.gs.idx = static_cast<const uint2*>(d[0]);

@@ -187,3 +187,42 @@ def test_footprint_is_what_a_plan_holds(host, C, n_dm):
     assert C < 1000 or any(c.startswith("gsum8") for c in host.configs(h))
     host.lib.dd_plan_info(h, None, None, ctypes.byref(held))
     assert sized.value == held.value
+
+
+@pytest.mark.parametrize("n_dm", [64, 600])
+def test_a_plan_without_room_for_grouped_sums_works_without_them(host, n_dm):
+    """Allocations failing one after another: the delay tables are needed, the
+    grouped-sum tables are not.  Nothing is left behind either way."""
+    i32, i64 = ctypes.c_int32, ctypes.c_int64
+    host.lib.dd_plan_info.argtypes = [ctypes.c_void_p, ctypes.POINTER(i64), ctypes.POINTER(i32), ctypes.POINTER(i64)]
+    host.lib.fake_fail_malloc.argtypes = [ctypes.c_long]
+    host.lib.fake_live.restype = ctypes.c_long
+    s = _apertif(20000, n_dm)
+    live = host.lib.fake_live()
+
+    def make(fail):
+        host.lib.fake_fail_malloc(fail)
+        h, held = ctypes.c_void_p(), i64()
+        status = host.lib.dd_plan(ctypes.byref(h), *s.plan_args(), U8)
+        host.lib.fake_fail_malloc(0)
+        if status != 0:
+            assert host.lib.fake_live() == live
+            return status, None, None, None
+        names, chosen = host.configs(h), host.selected(h)
+        host.lib.dd_plan_info(h, None, None, ctypes.byref(held))
+        assert len(host.forward(h)) == 1
+        host.lib.dd_plan_destroy(h)
+        assert host.lib.fake_live() == live
+        return 0, names, chosen, held.value
+
+    status, names, chosen, held = make(0)
+    shapes = [c for c in names if c.startswith("gsum8")]
+    assert status == 0 and chosen in shapes
+    for k in (1, 2, 3):                                  # delays, their transpose, the status word
+        assert make(k)[0] == 4, k                        # DD_ERR_NOMEM
+    for k in range(4, 4 + 2 * len(shapes)):              # two tables a shape
+        status, left, chosen_now, held_now = make(k)
+        missing = shapes[(k - 4) // 2]
+        assert status == 0, k
+        assert left == [c for c in names if c != missing] and chosen_now in left and held_now < held
+    assert make(4 + 2 * len(shapes)) == (0, names, chosen, held)
