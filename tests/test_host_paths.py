@@ -226,3 +226,13 @@ def test_a_plan_without_room_for_grouped_sums_works_without_them(host, n_dm):
         assert status == 0, k
         assert left == [c for c in names if c != missing] and chosen_now in left and held_now < held
     assert make(4 + 2 * len(shapes)) == (0, names, chosen, held)
+
+
+def test_the_adjoint_uses_shared_sums_where_it_is_tested(host):
+    """The sizes by which tests/test_gsum_gpu.py means to run float GSUM do."""
+    i64, vp = ctypes.c_int64, ctypes.c_void_p
+    host.lib.dd_adjoint.argtypes = [vp, vp, i64, vp, vp, i64, vp, i64, vp, vp]
+    for C, n_dm, n_out in [(1024, 70, 9001), (700, 64, 9000), (1019, 33, 12345), (1024, 2048, 20000)]:
+        h = host.plan(_apertif(n_out, n_dm, C), F32)
+        names = host.launches(lambda: host.lib.dd_adjoint(h, 4096, 1 << 40, None, 8192, 1 << 40, None, 0, None, None))
+        assert len(names) == 1 and "fwd_gsum_kernelIf" in names[0], (C, n_dm, n_out, names)
