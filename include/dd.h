@@ -118,7 +118,8 @@ dd_status dd_plan_destroy(dd_plan_t plan);
  * Sizes derived by the plan (any output pointer may be NULL):
  *   n_in         input samples per channel row that are read, n_out + max_delay;
  *   max_delay    the largest delay in samples (lowest channel, last DM trial);
- *   device_bytes device memory the plan holds (delay table + descriptors).
+ *   device_bytes device memory the plan holds (delay tables, descriptors, and
+ *                the grouped-sum tables of every uint8 shape it offers).
  */
 dd_status dd_plan_info(dd_plan_t plan, int64_t* n_in, int32_t* max_delay, int64_t* device_bytes);
 
@@ -138,8 +139,11 @@ dd_status dd_plan_in_stride(dd_plan_t plan, int64_t* in_row_stride);
  * Host-only sizing (no device memory is touched): the device bytes that
  * dd_plan of this geometry would hold (dd_plan_info's device_bytes of the
  * plan it makes: the delay table of Eq. 1, its transposed copy, the status
- * word and the window descriptors; n_out does not change it).  Arguments and
- * errors as dd_plan.  For admission control, e.g. a serving loop that keeps
+ * word, the window descriptors and the grouped-sum tables; n_out does not
+ * change it).  A plan made while the grouped-sum tables do not fit the device
+ * holds less: it is made without those.  The tables' sizes depend on the delays,
+ * so the call makes them on up to eight host threads, and frees them.
+ * Arguments and errors as dd_plan.  For admission control, e.g. a serving loop that keeps
  * beams within an HBM budget.
  */
 dd_status dd_plan_footprint(int32_t channels, double f_low_mhz, double chan_bw_mhz, double t_samp_s,
@@ -167,7 +171,8 @@ dd_status dd_plan_selected_config(dd_plan_t plan, int32_t* k);
 /*
  * Failure detection.  Every wait inside the library's kernels is bounded
  * (about one second); a wait that expires makes the kernel record a nonzero
- * code in the plan's device status word and return early instead of hanging.
+ * code in the plan's device status word and return early instead of hanging;
+ * the output of that launch is undefined.
  * This call waits for the device, reads that word into *code and clears it:
  * DD_OK if it was 0, DD_ERR_STATE otherwise (1 = a bounded wait expired).
  */
@@ -294,16 +299,17 @@ dd_status dd_boxcar_snr(const float* x, int64_t row_stride, int32_t n_rows, int6
  * fail) on its hot path, or a host framework that owns every device
  * allocation itself and does not let plug-ins allocate.  This call does the
  * same computation with the same arguments and results as dd_boxcar_snr but
- * allocates nothing: its per-row scratch lives in a fixed array inside the
- * library, DD_NOALLOC_MAX_ROWS rows of 32 bytes (2 MiB), which every GPU that
- * loads the library holds until the process exits.
+ * allocates nothing: with grad its per-row scratch is in the gradient's rows (as
+ * dd_boxcar_snr's), without it in a fixed array inside the library,
+ * DD_NOALLOC_MAX_ROWS rows of 32 bytes (2 MiB), which every GPU that loads the
+ * library holds until the process exits.
  *  - n_rows > DD_NOALLOC_MAX_ROWS is rejected with DD_ERR_SHAPE.
  *  - The first call on a device looks up that array's device address (once
  *    per device, with the device current); make that first call before any
  *    stream capture.  The address belongs to the device's context: after
  *    cudaDeviceReset (or anything else that replaces the context) the next
  *    call looks it up again, so that call too should come before any capture.
- *  - Every call on a device shares the one array and it keeps the previous
+ *  - Every call without grad on a device shares the one array and it keeps the previous
  *    call's contents; nothing in it needs to start at zero (each call writes
  *    every entry it reads).  Calls that can overlap on the GPU (different
  *    streams, or different host threads on the same device) race on it and

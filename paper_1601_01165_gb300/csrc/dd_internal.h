@@ -41,7 +41,7 @@ struct GsLaunch {
   const uint4* desc = nullptr;
   int desc_max = 0;             // bytes of the largest descriptor
   int padp = 0;                 // staged row pitch less the tile length
-  int cap = 0;                  // row elements of one of the two buffers
+  int cap = 0;                  // row elements of one of a block's row buffers (two to four)
   float patterns = 0;           // patterns per block and group, on average
   float samples = 0;            // samples of their rows, likewise
   int reach = 0;                // elements from a stage's start a leaf read may touch
@@ -57,12 +57,12 @@ struct TileConfig {
   Kind kind;
   int bd;       // DM trials per block
   int bt;       // output samples per block
-  int cc;       // channels per pipeline stage
-  int stages;   // pipeline depth
+  int cc;       // channels per pipeline stage (GSUM: row buffers)
+  int stages;   // pipeline depth (GSUM: groups of spans)
   int threads;  // threads per block
-  int spl;      // TMW6: samples per lane
+  int spl;      // TMW6, GSUM: samples per lane
   int smem;     // dynamic shared memory bytes (filled per plan)
-  int pitch;    // staged row pitch in elements (filled per plan)
+  int pitch;    // staged row pitch in elements (filled per plan; GSUM: summing warps)
   std::string name;
   GsLaunch gs{};  // GSUM (filled per plan)
 };

@@ -27,7 +27,7 @@
 // Rings of mbarriers join them (RB groups of rows); nothing in the group loop
 // is block-wide.
 //
-// What bounds it is shared memory (57 % of its cycles on uint8, 70 on float) and the
+// What bounds it is shared memory (57 % of its cycles on uint8, 68 on float) and the
 // chain of its reads in the row makers.  One Apertif uint8 beam (1024 x 2048 x
 // 20,000; u8pk takes 2.09 ms), each step measured: every warp making rows and
 // adding between two block barriers 3.7 ms (one warp's chain of dependent reads
@@ -319,7 +319,8 @@ struct Sums<uint8_t, DPW, SPL> {
 // groups; the sets take groups in turn, as the chain of reads that makes one
 // group's rows takes longer than adding them), NC add them up.  Every wait is
 // bounded; a warp whose wait ran out goes through its remaining groups
-// without waiting or working, and the block writes no output.
+// without waiting or working and stores nothing more.  It reports the timeout;
+// what the launch's output holds then is undefined (other warps store theirs).
 template <typename Tin, int NC, int NS, int NP, int DPW, int SPL, int SS, int RB, int MB>
 __global__ void __launch_bounds__(32 * (NC + NS * NP + 1), MB) fwd_gsum_kernel(FwdArgs a, GsLaunch gs) {
   using Row = typename GsTypes<Tin>::Row;

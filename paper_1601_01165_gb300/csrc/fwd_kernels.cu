@@ -757,8 +757,9 @@ static cudaError_t launch_naive(const TileConfig& cfg, const FwdArgs& a, cudaStr
 // Every row starts on 16 bytes: the form of a shared-memory kernel that need not
 // look where a row starts (on the Apertif uint8 beam 2.09 ms against 2.14).
 static bool rows16(const FwdArgs& a, int elem) { return a.in_stride * elem % 16 == 0; }
-// The other form exists for the shapes a plan chooses by itself (dd_plan.cpp);
-// an input whose rows do not start on 16 bytes goes to one of these.
+// The other form exists for most shapes a plan chooses by itself (dd_plan.cpp; not
+// for staged d8 t1024, d32 t384 and u8pk's 16-channel chunks); an input whose
+// rows do not start on 16 bytes goes to the one of them with the least estimate.
 static constexpr bool any_rows_staged(int bd, int bt, int cc) {
   return (bd == 8 && (bt == 256 || bt == 512)) || (bd == 16 && bt == 512) || (bd == 32 && bt == 512 && cc == 8);
 }

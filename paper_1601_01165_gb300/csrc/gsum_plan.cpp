@@ -13,7 +13,7 @@
 // The sum of a group is the sum of its two halves' (leaves 0-3 and 4-7), and
 // a half has few versions (relative delays of its own four leaves) in a block.
 // One descriptor, in 16-byte units:
-//   [0]            x = batches, y = row length, z = rows
+//   [0]            x = batches, y = row length
 //   [1 .. BD/4]    per trial: where its first sample is, in row elements
 //   then per batch of up to kGsVersions versions of the first half:
 //     x = versions of the first half in it, y = of the second half that occur
@@ -155,7 +155,7 @@ static void build_pairs(const dd_plan_s& p, int bd, int T, int padp, int64_t f0,
       t.desc[head] = uint4{(uint32_t)(v1 - v0), (uint32_t)n_second, 0, 0};
       ++n_batches;
     }
-    t.desc[at] = uint4{(uint32_t)n_batches, (uint32_t)row_len, (uint32_t)n_p, 0};
+    t.desc[at] = uint4{(uint32_t)n_batches, (uint32_t)row_len, 0, 0};
     t.idx.push_back(uint2{(uint32_t)at, (uint32_t)(t.desc.size() - at)});
     t.desc_max = std::max(t.desc_max, (int)(t.desc.size() - at) * 16);
   }

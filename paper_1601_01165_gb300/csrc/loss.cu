@@ -154,7 +154,7 @@ __device__ __forceinline__ void boxcars(const float* x, F visit) {
 // One block per row: mean, sd, best S/N and where it is; with ZERO the block
 // also clears the row of the gradient while it computes.
 //
-// Instruction issue bounds it (75 % of the slots; about 120 instructions a sample, where
+// Instruction issue bounds it (77 % of the slots; 144 instructions a sample, where
 // reading and clearing a 2048 x 20,000 block of 164 MB take 24 us each), so a
 // row is passed over twice with as little as each needs:
 //  1. the sum of the samples, which gives the boxcars' (a sample counts in
@@ -432,7 +432,8 @@ extern "C" dd_status dd_boxcar_snr(const float* x, int64_t row_stride, int32_t n
 }
 
 // ------------------------------------------------------ allocation-free form
-// Per-row scratch for dd_boxcar_snr_noalloc.  It is part of the library image,
+// Per-row scratch for dd_boxcar_snr_noalloc without a gradient (with one, the
+// statistics wait in its rows).  It is part of the library image,
 // so each GPU that loads the library carries it (2 MiB) until the process
 // exits, and no call ever has to allocate.  Host code cannot use the symbol
 // itself as a device address: the address is looked up per device below.
